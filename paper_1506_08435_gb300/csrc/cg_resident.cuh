@@ -1,0 +1,364 @@
+// The CG phase of mid-size solves with every vector but one on the SM.
+//
+// Pipelined CG (Ghysels & Vanroose, Parallel Comput. 40, 2014) on the face, as
+// form 2 of gpcg.cuh: the same recurrences, start and stop test.  What differs
+// is where things live and who waits.  A mid-size system gives an SM a few tens
+// of slices of 32 rows, whose operator is in shared memory (SellF64Local,
+// SellF32DiffLocal).  Here the block's rows of the nine CG vectors are there
+// too for the whole phase; only m = D^-1 w, which other rows gather, goes
+// through global memory, double-buffered.  (In registers, unrolled over a
+// thread's rows, they spilled from three rows a thread on.)
+//
+// What bounds an iteration on GB300 is latency: an FP64 warp instruction holds
+// its sub-core for 64 cycles whatever it adds up, so a block-wide sum over 16
+// warps, the division behind a coefficient and a grid barrier each cost as
+// much as the arithmetic of the pass.  Therefore
+//   * few compute warps with several slices each: a thread's rows are added by
+//     the dot products' own FMAs, and the tree over the block has 4-12 warps;
+//   * the two things that every block waits for are apart and hidden.  m goes
+//     out first and its barrier (counter count2, warp 12) runs while the other
+//     five recurrences and the dot products are computed; the sums and the
+//     scalar step (warps 13-15, counter count) run while the next product is
+//     computed, which needs m only.
+// The product of the iteration after the last one is thus computed and not
+// used (one per phase; it is counted).
+//
+// Measured against form 2 with 16 warps and the vectors in L2, us per product
+// of the whole solve: 50 x 50 6.4 -> 4.6, 120 x 120 6.4 -> 4.4, 397 x 283 10.2
+// -> 6.5, 30^3 7.6 -> 4.5, 44^3 11.8 -> 7.6, 50^3 12.6 -> 10.1; the 40^3
+// transient run, where every fourth product is a gradient projection's, 9.6 ->
+// 7.4 in FP64.  At 40^3 an iteration is 12,500 cycles: product 6,200, waiting
+// for the coefficients 1,200, recurrences and dot products 3,700, tree 700.
+//
+// Named barriers: 1 m written, 2 m visible grid-wide, 3 warp totals written,
+// 4 coefficients ready, 5 among the summing warps.
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+#include "team.cuh"
+#include "ops.cuh"
+
+namespace nnqp {
+
+constexpr int kResWarps = 12;         // compute warps at most; warps 12-15 serve (512-thread blocks)
+constexpr int kResVectors = 9;        // vectors of the block's rows in shared memory
+
+// Compute warps for at most `per` slices a block: 8 (two a sub-core) up to
+// three slices a warp, then 12; 4 where a warp has one slice at most.
+__host__ __device__ __forceinline__ int resident_warps(int64_t per) { return per <= 4 ? 4 : per <= 24 ? 8 : 12; }
+
+// x != 0 without a floating-point comparison (FP64 ones hold the FP64 unit).
+__device__ __forceinline__ bool is_set(double x) { return __double_as_longlong(x) != 0; }
+__device__ __forceinline__ bool is_set(float x) { return __float_as_int(x) != 0; }
+
+__device__ __forceinline__ void named_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+template <typename P>
+__device__ __forceinline__ P *in_shared(P *p) {
+    return (P *)__cvta_shared_to_generic(__cvta_generic_to_shared((const void *)p));
+}
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Whether the phase ends after update `it`, read by every warp behind barrier
+// 4.  The words are double-buffered by the update's parity: a warp that is
+// slow to read them must not meet those of the next update, or it would leave
+// alone and the block's barriers would no longer match.
+__device__ __forceinline__ bool resident_done(const RedSmem &sm, int it, int64_t left) {
+    const double *sc = sm.sc + 8 * (it & 1);
+    return flag_set(sc[0]) || flag_set(sc[4]) || !flag_set(sc[3]) || sm.flag2[it & 1] == 0 || it >= left;
+}
+
+// Products y = A x of the rows of a compute warp's slices (local slices warp,
+// warp + na, ... < ns).  The warp issues in order and 8 multiply-adds hold the
+// sub-core's FP64 unit for 512 cycles, so the gathers run two batches of 8
+// entries ahead of them: the next rows' loads are in flight while this row's
+// terms are added (measured at 40^3: 6,300 cycles per product with a row's
+// gathers issued at once and the next row's behind its multiply-adds).
+// done(l, a0, a1) takes the sums of local row l = 32 slice + lane.
+template <class Op, typename V, class FX, class F>
+__device__ __forceinline__ void resident_product(const Op &A, const int *sl, bool wide, int warp, int na, int ns,
+                                                 int lane, const V *x, FX &&xi, F &&done) {
+    V X0[8], X1[8];
+    auto width = [&](int t) { return t < ns ? (sl[t + 1] - sl[t]) >> 5 : 0; };
+    int t = warp, w = width(t);
+    if (!wide) {   // rows of at most 8 entries (2D meshes): one batch a slice
+        int w1 = width(t + na);
+        A.gather8(t < ns ? sl[t] : 0, w, 0, lane, x, X0);
+        A.gather8(w1 ? sl[t + na] : 0, w1, 0, lane, x, X1);
+        while (t < ns) {
+            V a0 = (V)0, a1 = (V)0;
+            A.fma8(sl[t], w, 0, lane, X0, xi(32 * t + lane), a0, a1);
+            const int t2 = t + 2 * na, w2 = width(t2);
+            A.gather8(w2 ? sl[t2] : 0, w2, 0, lane, x, X0);
+            done(32 * t + lane, a0, a1);
+            t += na;
+            if (t >= ns) break;
+            a0 = (V)0;
+            a1 = (V)0;
+            A.fma8(sl[t], w1, 0, lane, X1, xi(32 * t + lane), a0, a1);
+            const int t3 = t + 2 * na;
+            w = w2;
+            w1 = width(t3);
+            A.gather8(w1 ? sl[t3] : 0, w1, 0, lane, x, X1);
+            done(32 * t + lane, a0, a1);
+            t += na;
+        }
+        return;
+    }
+    if (t >= ns) return;
+    int off = sl[t];
+    A.gather8(off, w, 0, lane, x, X0);
+    A.gather8(off, w, 8, lane, x, X1);
+    for (;;) {
+        const int tn = t + na, wn = width(tn), offn = tn < ns ? sl[tn] : 0;
+        const V xl = xi(32 * t + lane);
+        V a0 = (V)0, a1 = (V)0;
+        A.fma8(off, w, 0, lane, X0, xl, a0, a1);
+        A.gather8(offn, wn, 0, lane, x, X0);
+        A.fma8(off, w, 8, lane, X1, xl, a0, a1);
+        for (int k = 16; k < w; k += 8) {
+            A.gather8(off, w, k, lane, x, X1);
+            A.fma8(off, w, k, lane, X1, xl, a0, a1);
+        }
+        A.gather8(offn, wn, 8, lane, x, X1);
+        done(32 * t + lane, a0, a1);
+        if (tn >= ns) break;
+        t = tn;
+        off = offn;
+        w = wn;
+    }
+}
+
+// One CG phase from v.x, v.g; leaves the step in v.s.  Every thread of every
+// block calls it; na compute warps.  Returns 0, ST_TIMEOUT when a wait gave
+// up, or 1 when the face has nothing to reduce.  A call of its own: the
+// registers the caller keeps live are saved once per phase.
+template <class Op, typename V>
+__device__ __noinline__ int cg_resident(GridTeam &T_, const Rows &R_, const Op &A_, const Bounds<V> &B,
+                                        const GpcgVecs<V> &v_, const GpcgCtl &C_, GpcgStats &st, double ftol2,
+                                        int na) {
+    GridTeam T = T_;
+    const Rows R = R_;
+    Op A = A_;
+    if constexpr (IsResidentOp<Op>::local) {
+        A.col = in_shared(A.col);   // (the compiler would read them with generic loads)
+        A.val = in_shared(A.val);
+    }
+    const GpcgVecs<V> v = v_;
+    const double eta2 = C_.eta2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool compute = warp < na;
+    RedSmem &sm = *in_shared(T.sm);
+    const V zero = (V)0;
+    const int ns = (int)(R.s1 - R.s0), nl = ns * 32, base = (int)(R.s0 * 32);
+    const int n = (int)(R.n - base) < nl ? (int)(R.n - base) : nl;   // local rows in use
+    V *const z = in_shared(v.res), *const q = z + nl, *const p = q + nl, *const s = p + nl, *const r = s + nl,
+            *const w = r + nl, *const u = w + nl, *const di = u + nl, *const y = di + nl;
+    int *const sl = in_shared(v.res_sl);   // [ns + 1] first entry of each local slice
+    V *mc = v.gw + base, *mn = v.m2 + base;
+    const int64_t e0 = __ldg(A.sptr + R.s0);   // entries are counted from the block's first
+    if constexpr (!IsResidentOp<Op>::local) {
+        A.col += e0;
+        A.val += e0;
+    }
+    for (int t = threadIdx.x; t <= ns; t += blockDim.x) sl[t] = (int)(__ldg(A.sptr + R.s0 + t) - (IsResidentOp<Op>::local ? A.e0 : e0));
+    // rows l = 32 t + lane of the slices t = warp, warp + na, ... belong to
+    // this thread throughout; a row off the face (or past the end) has di = 0
+    if (compute)
+#pragma unroll 1
+        for (int l = 32 * warp + lane; l < nl; l += 32 * na) {
+            V ri = zero, ui = zero, dl = zero;
+            if (l < n) {
+                const int64_t i = base + l;
+                const V xi = v.x[i];
+                if (xi > B.l(i) && xi < B.h(i)) {
+                    dl = v.dinv[i];
+                    ri = -v.g[i];
+                    ui = dl * ri;
+                }
+                mn[l] = ui;
+            }
+            z[l] = q[l] = p[l] = s[l] = zero;
+            r[l] = ri;
+            u[l] = ui;
+            di[l] = dl;
+        }
+    st.vec += 4;
+    st.fl += 1;
+    if (!T.sync()) return ST_TIMEOUT;
+    bool wide = false;
+    for (int t = threadIdx.x; t < ns; t += blockDim.x) wide = wide || sl[t + 1] - sl[t] > 8 * 32;
+    wide = __syncthreads_or(wide);
+    Acc<V> a3[2];
+    if (compute)
+        resident_product(
+            A, sl, wide, warp, na, ns, lane, mn - base, [&](int l) { return u[l]; },
+            [&](int l, V a0, V a1) {
+                const V dl = di[l], wl = is_set(dl) ? A.row_end(a0, a1, u[l], A.own(base + l, l < n), r[l]) : zero;
+                w[l] = wl;
+                if (l < n) mc[l] = dl * wl;
+                a3[0] += r[l] * u[l];
+                a3[1] += wl * u[l];
+            });
+    double d3[2], o3[7];
+    if (!team_sum_scalar(T, a3, d3, o3, [&](const double (&d)[2], double (&o)[7]) { cg_scalar_start(d, o); }))
+        return ST_TIMEOUT;
+    ++st.spmv;
+    st.fl += 6;
+    if (flag_set(o3[0])) {
+        __syncthreads();
+        T_ = T;
+        return 1;   // no step on this face
+    }
+    CgScalars cs;
+    cg_take(cs, o3);
+    // updates allowed: at least one, as in the other forms
+    int64_t left = C_.max_spmv - st.spmv;
+    if (left > C_.cg_max) left = C_.cg_max;
+    if (left < 1) left = 1;
+    const int n1 = na * 32 + 32, n4 = na * 32 + 128;
+    int it = 0;   // updates done
+    if (compute) {
+        V va = (V)cs.alpha, vb = (V)cs.beta;
+        for (;;) {
+            resident_product(
+                A, sl, wide, warp, na, ns, lane, mc - base, [&](int l) { return di[l] * w[l]; },
+                [&](int l, V a0, V a1) {
+                    const V dl = di[l];
+                    y[l] = is_set(dl) ? A.row_end(a0, a1, dl * w[l], A.own(base + l, l < n), w[l]) : zero;
+                });
+            if (it > 0) {
+                named_sync(4, n4);
+                if (resident_done(sm, it, left)) break;
+                va = (V)sm.sc[8 * (it & 1) + 1];
+                vb = (V)sm.sc[8 * (it & 1) + 2];
+            }
+#pragma unroll 1
+            for (int l = 32 * warp + lane; l < nl; l += 32 * na) {
+                const V wl = w[l], zl = y[l] + vb * z[l], wn = wl - va * zl;
+                z[l] = zl;
+                w[l] = wn;
+                y[l] = wl;   // w before the update, for q below
+                if (l < n) mn[l] = di[l] * wn;
+            }
+            __syncwarp();
+            named_arrive(1, n1);
+            Acc<V> a4[3];   // gamma, delta, r'r
+#pragma unroll 1
+            for (int l = 32 * warp + lane; l < nl; l += 32 * na) {
+                const V ql = y[l] + vb * q[l], pl = u[l] + vb * p[l];
+                const V rl = r[l] - va * ql, ul = di[l] * rl;
+                q[l] = ql;
+                p[l] = pl;
+                s[l] = s[l] + va * pl;
+                r[l] = rl;
+                u[l] = ul;
+                a4[0] += rl * ul;
+                a4[1] += w[l] * ul;
+                a4[2] += rl * rl;
+            }
+            double d4[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) d4[k] = a4[k].value();
+            warp_stage<3>(d4, sm);
+            __syncwarp();
+            named_arrive(3, n1);
+            ++it;
+            V *t = mc;
+            mc = mn;
+            mn = t;
+            named_sync(2, n1);
+        }
+#pragma unroll 1
+        for (int l = 32 * warp + lane; l < n; l += 32 * na) v.s[base + l] = s[l];
+    } else if (warp == kResWarps) {
+        // m of every block visible
+        for (;;) {
+            named_sync(1, n1);
+            ++it;
+            if (lane == 0) sm.flag2[it & 1] = T.arrive_and_wait_on(&T.bar->count2, T.wait2 + it);
+            __syncwarp();
+            named_arrive(2, n1);
+            named_sync(4, n4);
+            if (resident_done(sm, it, left)) break;
+        }
+    } else if (warp > kResWarps) {
+        // sums over the block, then over the grid (entry k by warp 13 + k); then
+        // the scalar step of cg_scalar_step, its two divisions and the stop test
+        // on a warp (and sub-core) each: warp 13 alpha, 14 beta and 1 / gamma,
+        // 15 the test.  (One warp after the other it took 1,850 cycles.)
+        const int k = warp - (kResWarps + 1);
+        int slot = T.slot;
+        double t = cs.igamma * cs.ialpha;                          // warp 13
+        double ig = cs.igamma;                                     // warp 14
+        double dec = 0.5 * cs.alpha * cs.gamma, maxdec = dec;      // warp 15
+        for (;;) {
+            slot ^= 1;
+            ++it;
+            double *P = T.partials + (size_t)slot * kMaxRed * T.nblocks;
+            double *sc = sm.sc + 8 * (it & 1);
+            if (k == 0) {
+                named_sync(3, n1);
+                warp0_sum_warps<3>(sm, na);
+                __syncwarp();
+                if (lane < 3) P[(size_t)lane * T.nblocks + blockIdx.x] = sm.bcast[lane];
+                __syncwarp();
+                if (lane == 0) sm.flag = T.arrive_and_wait_on(&T.bar->count, T.wait_id + it);
+                __syncwarp();
+            }
+            named_sync(5, 96);
+            const double sum = sm.flag ? sum_partials(P + (size_t)k * T.nblocks, T.nblocks) : 0.0;
+            if (lane == 0) sm.bcast[8 + k] = sum;
+            named_sync(5, 96);
+            const double gamma = sm.bcast[8];
+            double den = 0.0;
+            if (k == 0) {
+                den = fma(-gamma * gamma, t, sm.bcast[9]);         // delta - beta gamma / alpha
+                const double an = gamma / den;
+                if (lane == 0) {
+                    sc[1] = an;
+                    sc[4] = den > 0.0 ? 0.0 : 1.0;
+                }
+            } else if (k == 1) {
+                const double bn = gamma * ig;
+                ig = 1.0 / gamma;
+                if (lane == 0) {
+                    sc[2] = bn;
+                    sc[5] = ig;
+                }
+            } else {
+                const bool stop = dec <= eta2 * maxdec || sum <= ftol2 || !(gamma > 0.0);
+                if (lane == 0) {
+                    sc[0] = stop ? 1.0 : 0.0;
+                    sc[3] = sm.flag ? 1.0 : 0.0;
+                }
+            }
+            __syncwarp();
+            named_sync(4, n4);
+            if (resident_done(sm, it, left)) break;
+            if (k == 0) {
+                t = (den * sc[5]) * sc[5];
+            } else if (k == 2) {
+                dec = 0.5 * sc[1] * gamma;
+                maxdec = dec > maxdec ? dec : maxdec;
+            }
+        }
+        if (k == 0 && lane == 0) sm.its = flag_set(sm.sc[8 * (it & 1) + 3]) && sm.flag2[it & 1] ? it : -1;
+    }
+    __syncthreads();
+    it = sm.its;
+    if (it < 0) return ST_TIMEOUT;
+    T_ = T;
+    T_.slot ^= it & 1;
+    T_.wait_id += it;
+    T_.wait2 += it;
+    st.spmv += it + 1;
+    st.cg += it;
+    st.fl += 20 * (int64_t)it;
+    return 0;
+}
+
+}  // namespace nnqp

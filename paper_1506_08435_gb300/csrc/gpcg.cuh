@@ -208,6 +208,8 @@ struct GpcgVecs {
     uint8_t *fm;          // face mask of the current CG phase (1 = free)
     V *m2;                // second product input of the pipelined CG (variant 2)
     const SsorF64 *pc;    // SSOR ordering of the textbook form with CGV = 3 (else unused)
+    V *res;               // shared memory of the resident CG phase: kResVectors vectors of the block's rows,
+    int *res_sl;          //    and the first entries of its slices
 };
 
 struct GpcgCtl {
@@ -224,6 +226,8 @@ struct GpcgCtl {
                          //    reduction in one pass; needs GpcgVecs::m2)
     int keep_p;          // 1: the packed direction pass stores p with an L2 evict-last policy
                          //    (the product gathers it next, while its operator streams past)
+    int res_warps;       // form 2: compute warps of the CG phase with its vectors in shared memory
+                         //    (cg_resident.cuh), 0 = vectors in global memory
     int cg_bound_stop;   // 1: end the CG phase as soon as x + s leaves the box;
                          // 0: run CG to its stall test, the projected search clips
 };
@@ -237,6 +241,10 @@ struct GpcgStats {
     int64_t pc = 0;   // SSOR applications (their traffic is counted apart from vec)
     double gp2 = 0.0;
 };
+
+template <class Op, typename V>
+__device__ __noinline__ int cg_resident(GridTeam &T, const Rows &R, const Op &A, const Bounds<V> &B,
+                                        const GpcgVecs<V> &v, const GpcgCtl &C, GpcgStats &st, double ftol2, int na);
 
 // Runs GPCG from the iterate in v.x (projected first).  On exit v.x holds
 // the final iterate, v.g its gradient (pointers may have been swapped).
@@ -360,8 +368,15 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
         if (st.gp2 <= tol2 || st.spmv >= C.max_spmv || !isfinite(st.gp2)) continue;
         // ------------------------------------------------ CG on faces
         const bool count_cross = C.cg_bound_stop != 0;
+        constexpr bool can_reside = CGV == 2 && IsResidentOp<Op>::value && IsGridTeam<Team>::value;
         for (;;) {
-            if ((CGV >= 0 ? CGV : C.cg_variant) == 1) {
+            if (can_reside && C.res_warps > 0) {
+                if constexpr (can_reside) {
+                    const int e = cg_resident(T, R, A, B, v, C, st, ftol2, C.res_warps);
+                    if (e == ST_TIMEOUT) return ST_TIMEOUT;
+                    if (e != 0) break;
+                }
+            } else if ((CGV >= 0 ? CGV : C.cg_variant) == 1) {
                 // Chronopoulos-Gear form: one fused reduction per iteration
                 // (gamma = r'u and delta = w'u with u = D^-1 r, w = A_F u), the
                 // product A p carried by the recurrence q = w + beta q.
@@ -762,3 +777,5 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
 }
 
 }  // namespace nnqp
+
+#include "cg_resident.cuh"

@@ -76,6 +76,8 @@ struct GridArgs {
     uint8_t *fmask;         // [n] face mask of the CG phases
     int tma_slot_entries;   // FMT 3: 32 x the widest slice (slot size of the streamed operator)
     int tma_slots;          // FMT 3: slots per warp
+    int res_offset;         // where the resident CG phase's shared memory begins (its slice table first)
+    int res_table;          // bytes of that table
     SsorF64 pc;             // SSOR ordering and omega (CG form 3, TRON with ncolors > 0)
 };
 
@@ -160,10 +162,15 @@ template <int FMT, int MODE, int CGV, int TPB>
 __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k_solve_grid(GridArgs a) {
     __shared__ RedSmem sm;
     extern __shared__ __align__(16) unsigned char op_smem[];
-    GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm};
+    GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm, 0, 0};
     const Rows R = rows_of_block(a.n, a.nslices, blockIdx.x, gridDim.x);
+    // the SSOR sweeps spread a colour over every warp of the grid
+    T.active = CGV == 3 ? TPB / 32 : R.active_warps(TPB / 32);
     double *x = a.v64[0];
     R.each([&](int64_t i) { x[i] = a.c_in[a.free_node[i]]; });
+    // shared memory of the resident CG phase (behind the operator of FMT 2)
+    constexpr bool RES = CGV == 2 && TPB == 512 && (FMT == 2 || FMT == 0);
+    unsigned char *res = op_smem + a.res_offset;
     SellF64Local Aloc{};
     SellF32DiffLocal A32loc{};
     SellF32DiffTma A32tma{};
@@ -218,6 +225,10 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k
                               a.v32[6], a.v32[7], a.v32[8], a.v32[9], a.dinv32, a.fmask, a.v32[12]};
             GpcgVecs<double> v64{x, a.v64[1], a.v64[2], a.v64[3], a.v64[4], a.v64[5],
                                  a.v64[6], a.v64[7], a.v64[8], b, a.dinv64, a.fmask, a.v64[10]};
+            if constexpr (RES) {
+                v.res_sl = reinterpret_cast<int *>(res);
+                v.res = reinterpret_cast<float *>(res + a.res_table);
+            }
             MixedStats ms;
             if constexpr (FMT == 2)
                 status = mixed_solve<CGV, inner_cg_form(MODE, CGV), true>(T, R, a.A, A32loc, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
@@ -227,7 +238,13 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k
                 status = mixed_solve<CGV, inner_cg_form(MODE, CGV), (TPB < 512)>(T, R, a.A, A32tma, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
                                                  a.v32[11], v64, a.rtol * den, a.inner_rtol, a.max_ref,
                                                  a.ctl.max_spmv, a.inner_cap, a.ctl, a.ctl, ms);
-            else
+            else if constexpr (RES) {
+                SellF32DiffRes A32r;
+                static_cast<SellF32Diff &>(A32r) = a.A32;
+                status = mixed_solve<CGV, inner_cg_form(MODE, CGV), true>(T, R, a.A, A32r, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
+                                                 a.v32[11], v64, a.rtol * den, a.inner_rtol, a.max_ref,
+                                                 a.ctl.max_spmv, a.inner_cap, a.ctl, a.ctl, ms);
+            } else
                 status = mixed_solve<CGV, inner_cg_form(MODE, CGV), true>(T, R, a.A, a.A32, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
                                                  a.v32[11], v64, a.rtol * den, a.inner_rtol, a.max_ref,
                                                  a.ctl.max_spmv, a.inner_cap, a.ctl, a.ctl, ms);
@@ -248,12 +265,20 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k
                                a.v64[6], a.v64[7], a.v64[8], b, a.dinv64, a.fmask, a.v64[10]};
             const SsorF64 pcv = a.pc;
             if constexpr (CGV == 3) v.pc = &pcv;
+            if constexpr (RES) {
+                v.res_sl = reinterpret_cast<int *>(res);
+                v.res = reinterpret_cast<double *>(res + a.res_table);
+            }
             GpcgCtl c = a.ctl;
             c.tol = a.rtol * den;
             c.face_tol = 0.5 * c.tol;
             GpcgStats gs;
             const Bounds<double> B{a.lo, a.hi, nullptr, nullptr};
-            if constexpr (FMT == 0)
+            if constexpr (FMT == 0 && RES) {
+                SellF64Res Ar;
+                static_cast<SellF64 &>(Ar) = a.A;
+                status = gpcg_solve<GridTeam, SellF64Res, double, CGV>(T, R, Ar, B, v, c, gs);
+            } else if constexpr (FMT == 0)
                 status = gpcg_solve<GridTeam, SellF64, double, CGV>(T, R, a.A, B, v, c, gs);
             else if constexpr (FMT == 2)
                 status = gpcg_solve<GridTeam, SellF64Local, double, CGV>(T, R, Aloc, B, v, c, gs);

@@ -110,6 +110,37 @@ struct SellF64X {
         return a0 + a1;
     }
 
+    // Pieces of a row's product for the resident CG phase (cg_resident.cuh):
+    // the gathers of entries k .. k + 7 of a row of width w (off = base - e0),
+    // and their multiply-adds.
+    __device__ __forceinline__ void gather8(int off, int w, int k, int lane, const double *x, double (&xv)[8]) const {
+        const int2 *c2 = reinterpret_cast<const int2 *>(col + off) + lane + 16 * k;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k + 2 * j < w) {
+                const int2 c = mat_load<LOCAL>(c2 + 32 * j, stream);
+                xv[2 * j] = x[c.x];
+                xv[2 * j + 1] = x[c.y];
+            }
+    }
+    __device__ __forceinline__ void fma8(int off, int w, int k, int lane, const double (&xv)[8], double, double &a0,
+                                         double &a1) const {
+        const double2 *v2 = reinterpret_cast<const double2 *>(val + off) + lane + 16 * k;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k + 2 * j < w) {
+                const double2 v = mat_load<LOCAL>(v2 + 32 * j, stream);
+                a0 = fma(v.x, xv[2 * j], a0);
+                a1 = fma(v.y, xv[2 * j + 1], a1);
+            }
+    }
+    // The gathered vector is D^-1 y; yi, y's entry of the row, is therefore
+    // the row's diagonal term (x_i and own(): the FP32 operator's).
+    __device__ __forceinline__ double own(int64_t, bool) const { return 0.0; }
+    __device__ __forceinline__ static double row_end(double a0, double a1, double, double, double yi) {
+        return (a0 + yi) + a1;
+    }
+
     template <class Epi>
     __device__ __forceinline__ void apply(const Rows &R, const double *x, Epi &&epi) const {
         const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -153,6 +184,34 @@ struct SellF32DiffX {
     const float *__restrict__ rsum;
     bool stream = false;          // operator larger than L2: streaming loads + slice prefetch
     int64_t e0 = 0;               // first entry held by col/val (LOCAL)
+
+    // As SellF64X's, in difference form: xi = x of the row itself, d = own(i)
+    // its row sum s_i.
+    __device__ __forceinline__ void gather8(int off, int w, int k, int lane, const float *x, float (&xv)[8]) const {
+        const int2 *c2 = reinterpret_cast<const int2 *>(col + off) + lane + 16 * k;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k + 2 * j < w) {
+                const int2 c = mat_load<LOCAL>(c2 + 32 * j, stream);
+                xv[2 * j] = x[c.x];
+                xv[2 * j + 1] = x[c.y];
+            }
+    }
+    __device__ __forceinline__ void fma8(int off, int w, int k, int lane, const float (&xv)[8], float xi, float &a0,
+                                         float &a1) const {
+        const float2 *v2 = reinterpret_cast<const float2 *>(val + off) + lane + 16 * k;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k + 2 * j < w) {
+                const float2 v = mat_load<LOCAL>(v2 + 32 * j, stream);
+                a0 = fmaf(v.x, xv[2 * j] - xi, a0);
+                a1 = fmaf(v.y, xv[2 * j + 1] - xi, a1);
+            }
+    }
+    __device__ __forceinline__ float own(int64_t i, bool in) const { return in ? __ldg(rsum + i) : 0.0f; }
+    __device__ __forceinline__ static float row_end(float a0, float a1, float xi, float d, float) {
+        return fmaf(d, xi, a0 + a1);
+    }
 
     template <class Epi>
     __device__ __forceinline__ void apply(const Rows &R, const float *x, Epi &&epi) const {
@@ -337,12 +396,41 @@ struct SellF32DiffTma {
     }
 };
 
+// The operators of kernels whose CG phase keeps its vectors in shared memory
+// (cg_resident.cuh): in shared memory themselves, or, as these two, read from
+// global memory (the same entries in the same order: the results are the same
+// bits).
+struct SellF64Res : SellF64X<false> {};
+struct SellF32DiffRes : SellF32DiffX<false> {};
+template <class Op>
+struct IsResidentOp {
+    static constexpr bool value = false;
+};
+template <>
+struct IsResidentOp<SellF64X<true>> {
+    static constexpr bool value = true, local = true;
+};
+template <>
+struct IsResidentOp<SellF32DiffX<true>> {
+    static constexpr bool value = true, local = true;
+};
+template <>
+struct IsResidentOp<SellF64Res> {
+    static constexpr bool value = true, local = false;
+};
+template <>
+struct IsResidentOp<SellF32DiffRes> {
+    static constexpr bool value = true, local = false;
+};
+
 // Whether an operator streams through L2 (large systems): the vector passes
 // of its solves prefetch their next slices too.
 template <bool L>
 __device__ __forceinline__ bool op_streams(const SellF64X<L> &A) { return A.stream; }
 template <bool L>
 __device__ __forceinline__ bool op_streams(const SellF32DiffX<L> &A) { return A.stream; }
+__device__ __forceinline__ bool op_streams(const SellF64Res &A) { return A.stream; }
+__device__ __forceinline__ bool op_streams(const SellF32DiffRes &A) { return A.stream; }
 __device__ __forceinline__ bool op_streams(const SellF32DiffTma &) { return true; }
 template <class Op>
 __device__ __forceinline__ bool op_streams(const Op &) { return false; }

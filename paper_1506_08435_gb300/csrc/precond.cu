@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256) k_precond_apply(PcArgs a) {
             a.z[i] = (a.fm == nullptr || a.fm[i]) ? a.dinv[i] * a.r[i] : 0.0;
         return;
     }
-    GridTeam T{a.bar, nullptr, (int)gridDim.x, a.timeout_ns, 0, 0, &sm};
+    GridTeam T{a.bar, nullptr, (int)gridDim.x, a.timeout_ns, 0, 0, &sm, (int)(blockDim.x >> 5), 0};
     ssor_apply(T, a.S, a.fm, a.dinv, a.r, a.y, a.z, [](int64_t, double) {});
 }
 

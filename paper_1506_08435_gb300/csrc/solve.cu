@@ -18,8 +18,9 @@ namespace nnqp {
 __global__ void __launch_bounds__(kSolveThreads) k_lbfgs_grid(GridArgs a) {
     __shared__ RedSmem sm;
     __shared__ LbSmem lsm;
-    GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm};
+    GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm, 0, 0};
     const Rows R = rows_of_block(a.n, a.nslices, blockIdx.x, gridDim.x);
+    T.active = R.active_warps(blockDim.x >> 5);
     double *x0 = a.v64[0];
     R.each([&](int64_t i) { x0[i] = a.c_in[a.free_node[i]]; });
     if (!T.sync()) return;
@@ -54,8 +55,9 @@ __global__ void __launch_bounds__(kSolveThreads) k_lbfgs_grid(GridArgs a) {
 // The same driver with the trust-region Newton solver (FP64, SELL).
 __global__ void __launch_bounds__(kSolveThreads, 2) k_tron_grid(GridArgs a) {
     __shared__ RedSmem sm;
-    GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm};
+    GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm, 0, 0};
     const Rows R = rows_of_block(a.n, a.nslices, blockIdx.x, gridDim.x);
+    T.active = a.pc.ncolors > 0 ? (int)(blockDim.x >> 5) : R.active_warps(blockDim.x >> 5);
     double *x0 = a.v64[0];
     R.each([&](int64_t i) { x0[i] = a.c_in[a.free_node[i]]; });
     if (!T.sync()) return;
@@ -182,6 +184,9 @@ namespace {
 constexpr double kStreamBytes = 48.0 * (1 << 20);
 // Most shared memory a block's staged operator slices may take.
 constexpr size_t kSmemOperatorBytes = 192 * 1024;
+// ... and it together with the vectors of the resident CG phase (the block's
+// static shared memory takes another 11 KB of the 227).
+constexpr size_t kSmemBytes = 214 * 1024;
 // Shared-memory budget of the streamed FP32 operator's slots per block: one
 // 768-thread block per SM, 24 warps x 2 slots of 32 rows x up to 16 entries
 // x 8 bytes, plus a 2 KB header.
@@ -443,7 +448,14 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     // operator (the only one built at that size; below, the 512-thread
     // load-based kernel where the streamed operator does not apply).
     const bool large = !driver && (slices > (int64_t)4 * 8 * sms || force_large);
-    if (!driver && slices <= (int64_t)4 * 8 * sms && slices > (int64_t)8 * sms / 2) tpb = 512;
+    // The pipelined CG form of those systems keeps its vectors on the SM
+    // (cg_resident.cuh) in 512-thread blocks, which the smallest systems gain
+    // from as well (50 x 50: 5.3 ms in 19 blocks of 256 threads, 3.9 ms here);
+    // their slices are spread one to a block as far as there are SMs (12 to 76
+    // blocks measure alike there).
+    const bool mid = !driver && !large && slices <= (int64_t)4 * 8 * sms;
+    const bool on_chip = mid && fmt == NN_FMT_SELL && a.ctl.cg_variant == 2 && mode != MODE_MIXED;
+    if (mid && (on_chip || slices > (int64_t)8 * sms / 2)) tpb = 512;
     if (!driver && (force_tpb == 256 || force_tpb == 512)) tpb = force_tpb;
     if (large && (a.ctl.cg_variant == 0 || a.ctl.cg_variant == 3) && fmt == NN_FMT_SELL && force_tpb != 512)
         tpb = kLargeThreads;
@@ -479,17 +491,19 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     // rather than filling fewer blocks' warps (measured: 40^3 transient on
     // 131 -> 152 blocks 55.8 -> 52.3 ms; 50^2 steady on 10 -> 19 blocks
     // 3.72 -> 3.36 ms)
-    const int64_t spread = std::max<int64_t>(by_rows, (slices + 3) / 4);
+    const int64_t spread = on_chip && tpb == 512 ? slices : std::max<int64_t>(by_rows, (slices + 3) / 4);
     int want = (int)std::min<int64_t>(spread, slices <= (int64_t)4 * 8 * sms ? (int64_t)sms : (int64_t)maxg);
     want = std::min(want, maxg);
     if (large) want = maxg;
     if (o->grid_blocks > 0) want = std::min(o->grid_blocks, maxg);
     want = std::max(want, 1);
     // Mid-size SELL solves keep each block's slices of the operator of the
-    // inner products in shared memory when they fit (one block per SM).
+    // inner products in shared memory when they fit (one block per SM), and
+    // the vectors of their pipelined CG phase (cg_resident.cuh).
     size_t dyn_smem = 0;
     const char *sm_env = getenv("NNQP_SMEM_OP");
-    if (!driver && fmt == NN_FMT_SELL && tpb == 512 && !(sm_env && sm_env[0] == '0')) {
+    const bool smem_op = !(sm_env && sm_env[0] == '0');
+    if (!driver && fmt == NN_FMT_SELL && tpb == 512) {
         if (s->sptr_host.empty()) {
             s->sptr_host.resize((size_t)slices + 1);
             NN_CUDA_TRY(cudaMemcpyAsync(s->sptr_host.data(), s->A64.sptr, sizeof(int64_t) * (slices + 1),
@@ -502,19 +516,31 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
             const Rows rb = rows_of_block(n, slices, b, want);
             most = std::max(most, s->sptr_host[(size_t)rb.s1] - s->sptr_host[(size_t)rb.s0]);
         }
-        const size_t bytes = (size_t)most * (4 + vbytes);
-        GridKernel ks = grid_kernel(mode, FMT_SELL_SMEM, a.ctl.cg_variant, tpb);
+        const int64_t deep = (slices + want - 1) / want;   // slices of a block at most
+        const size_t op = (size_t)most * (4 + vbytes), table = ((size_t)(deep + 1) * 4 + 15) / 16 * 16;
+        const size_t vecs = table + (size_t)kResVectors * deep * 32 * vbytes;
+        const char *rw = getenv("NNQP_RES_WARPS");
+        const bool form = a.ctl.cg_variant == 2 && !a.ctl.cg_bound_stop && mode != MODE_MIXED && !(rw && atoi(rw) < 1);
+        const bool both = form && op + vecs <= kSmemBytes;
+        // (the resident phase is the same with either operator: whether it is
+        // taken does not depend on NNQP_SMEM_OP)
+        const bool resident = both || (form && op > kSmemOperatorBytes && vecs <= kSmemBytes);
+        const bool local = smem_op && op > 0 && (resident ? both : op <= kSmemOperatorBytes);
+        const size_t bytes = (local ? op : 0) + (resident ? vecs : 0);
+        GridKernel ks = bytes ? grid_kernel(mode, local ? FMT_SELL_SMEM : NN_FMT_SELL, a.ctl.cg_variant, tpb) : nullptr;
         // the attribute is set to the same budget by every caller (solves on
         // other host threads may launch this kernel at the same time)
-        if (ks && bytes > 0 && bytes <= kSmemOperatorBytes &&
-            cudaFuncSetAttribute((const void *)ks, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemOperatorBytes) == cudaSuccess) {
+        if (ks && cudaFuncSetAttribute((const void *)ks, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kSmemBytes) == cudaSuccess) {
             int per = 0;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ks, tpb, bytes);
             if (per * sms >= want) {
                 kern = ks;
                 dyn_smem = bytes;
                 maxg = per * sms;
+                a.ctl.res_warps = !resident ? 0 : rw ? std::min(atoi(rw), kResWarps) : resident_warps(deep);
+                a.res_offset = local ? (int)op : 0;
+                a.res_table = (int)table;
             }
         }
         cudaGetLastError();   // a refused attribute leaves the plain kernel in use

@@ -22,6 +22,8 @@ struct GridBarrier {
     unsigned long long count;     // arrivals since launch (never reset)
     int error;                    // 0 = fine, else an nn_status code
     int where;                    // diagnostic: id of the wait that gave up
+    unsigned long long pad[14];   // (the second counter on a 128-byte line of its own)
+    unsigned long long count2;    // arrivals of the resident CG phase's vector barrier
 };
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p) {
@@ -58,6 +60,8 @@ struct RedSmem {
     double bcast[kMaxRed];
     double sc[16];                // results of scalar steps done by warp 0
     int flag;
+    int flag2[2];                 // the vector barrier passed, by parity (resident CG phase)
+    int its;                      // updates of the resident CG phase, -1 = a wait gave up
 };
 
 // Warp stage of a block sum: K values per lane are summed over the warp's 32
@@ -148,23 +152,25 @@ __device__ __forceinline__ void warp_stage(const double (&v)[K], RedSmem &sm) {
     }
 }
 
-// Cross-warp stage: the per-warp totals sm.warp[w][k] (w < nw) are summed in
-// a fixed butterfly order by warp 0 and stored to sm.bcast[k].  Lanes are
-// packed (k, w) so that one FP64 instruction serves 32 / nw entries.
-// A block whose warp count is not a power of two (24 warps of 768 threads)
-// is summed as the next power of two with zero totals for the missing warps.
+// Cross-warp stage: the per-warp totals sm.warp[w][k] (w < nw) are summed by
+// the calling warp and stored to sm.bcast[k].  An FP64 warp instruction takes
+// 64 cycles of its sub-core whatever its active lanes (measured), an addition
+// behind a shuffle 118, so the lanes are packed for few dependent additions: L
+// lanes per entry, each adding every L-th warp's total, then log2 L shuffles
+// (16 warps: K <= 4 one addition and three shuffles for all entries, K <= 8
+// three and two; packing 32 / nw entries per instruction took 8 and 12).
 template <int K>
-__device__ __forceinline__ void warp0_sum_warps(RedSmem &sm) {
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    int np = 1;
-    while (np < nw) np <<= 1;
-    const int per = 32 / np;                  // entries per warp instruction
-    const int k_in = lane / np, w = lane % np;
-    for (int k0 = 0; k0 < K; k0 += per) {
-        const int k = k0 + k_in;
-        double t = (k < K && k_in < per && w < nw) ? sm.warp[w][k] : 0.0;
-        for (int o = np >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (w == 0 && k < K && k_in < per) sm.bcast[k] = t;
+__device__ __forceinline__ void warp0_sum_warps(RedSmem &sm, int nw) {
+    constexpr int P = K <= 4 ? 4 : K <= 8 ? 8 : K <= 16 ? 16 : 32;
+    constexpr int L = 32 / P;
+    const int lane = threadIdx.x & 31, j = lane % L;
+    for (int k0 = 0; k0 < K; k0 += P) {
+        const int k = k0 + lane / L;
+        double t = (k < K && j < nw) ? sm.warp[j][k] : 0.0;
+        for (int w = j + L; w < nw; w += L) t += k < K ? sm.warp[w][k] : 0.0;
+#pragma unroll
+        for (int o = L >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (j == 0 && k < K) sm.bcast[k] = t;
     }
 }
 
@@ -174,7 +180,7 @@ template <int K>
 __device__ __forceinline__ void block_sum(double (&v)[K], RedSmem &sm) {
     warp_stage<K>(v, sm);
     __syncthreads();
-    if ((threadIdx.x >> 5) == 0) warp0_sum_warps<K>(sm);
+    if ((threadIdx.x >> 5) == 0) warp0_sum_warps<K>(sm, blockDim.x >> 5);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < K; ++k) v[k] = sm.bcast[k];
@@ -195,6 +201,29 @@ struct BlockTeam {
     __device__ __forceinline__ bool ok() const { return true; }
 };
 
+// Sum of the nblocks per-block partials Pk by one warp, in a fixed order; the
+// result on every lane.  Up to 8 partials per lane per round, all loads
+// issued before the adds (one L2 round trip per 256 blocks).
+__device__ __forceinline__ double sum_partials(const double *Pk, int nblocks) {
+    const int lane = threadIdx.x & 31;
+    double u = 0.0;
+    for (int b0 = 0; b0 < nblocks; b0 += 256) {
+        double w[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int b = b0 + lane + 32 * j;
+            w[j] = b < nblocks ? __ldcg(Pk + b) : 0.0;
+        }
+        // (one block per SM needs five terms: each addition is 64 cycles)
+        double t = (w[0] + w[1]) + (w[2] + w[3]);
+        t += nblocks - b0 > 160 ? (w[4] + w[5]) + (w[6] + w[7]) : w[4];
+        u = b0 ? u + t : t;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+    return u;
+}
+
 struct GridTeam {
     GridBarrier *bar;
     double *partials;             // [2][kMaxRed][nblocks]
@@ -203,6 +232,8 @@ struct GridTeam {
     int slot;
     int wait_id;
     RedSmem *sm;
+    int active;                   // warps of this block that own rows: the others contribute nothing
+    int wait2;                    // vector barriers passed (count2; the resident CG phase)
 
     // Grid-wide barrier.  Every block knows how many barriers it has passed
     // (wait_id), so the k-th barrier is complete once the arrival counter
@@ -210,15 +241,16 @@ struct GridTeam {
     // (its block's writes become visible first) and polls the counter with
     // acquire loads, for at most timeout_ns; a wait that runs out sets the
     // error word, and a block that sees the error word set leaves as well.
-    // Arrival and bounded wait of the barrier numbered wait_id, by thread 0
+    // Arrival and bounded wait of the barrier numbered wait_id, by one thread
     // of the block (after the block's writes it must publish); 1 = passed.
-    __device__ int arrive_and_wait() {
+    __device__ int arrive_and_wait() { return arrive_and_wait_on(&bar->count, wait_id); }
+    __device__ int arrive_and_wait_on(unsigned long long *count, int id) {
         int ok = 1;
-        const unsigned long long target = (unsigned long long)wait_id * (unsigned long long)nblocks;
-        red_release_add_u64(&bar->count, 1ULL);
+        const unsigned long long target = (unsigned long long)id * (unsigned long long)nblocks;
+        red_release_add_u64(count, 1ULL);
         unsigned spins = 0;
         unsigned long long t0 = 0;
-        while (ld_acquire_u64(&bar->count) < target) {
+        while (ld_acquire_u64(count) < target) {
             ++spins;
             if ((spins & 63u) == 0) {
                 if (ld_relaxed_i32(&bar->error)) {
@@ -229,7 +261,7 @@ struct GridTeam {
                 if (t0 == 0) {
                     t0 = now;
                 } else if (now - t0 > timeout_ns) {
-                    if (atomicCAS(&bar->error, 0, 7 /* NN_ERR_TIMEOUT */) == 0) bar->where = wait_id;
+                    if (atomicCAS(&bar->error, 0, 7 /* NN_ERR_TIMEOUT */) == 0) bar->where = id;
                     ok = 0;
                     break;
                 }
@@ -250,7 +282,7 @@ struct GridTeam {
     template <int K>
     __device__ bool reduce(double (&v)[K]) {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        warp_stage<K>(v, *sm);
+        if (warp < active) warp_stage<K>(v, *sm);
         __syncthreads();
         slot ^= 1;
         ++wait_id;
@@ -258,7 +290,7 @@ struct GridTeam {
         // warp 0 sums the warps, publishes the block's partials and passes
         // the grid barrier; the other warps wait for it at one block barrier
         if (warp == 0) {
-            warp0_sum_warps<K>(*sm);
+            warp0_sum_warps<K>(*sm, active);
             __syncwarp();
             for (int k = lane; k < K; k += 32) P[(size_t)k * nblocks + blockIdx.x] = sm->bcast[k];
             __syncwarp();
@@ -270,21 +302,7 @@ struct GridTeam {
             // warp k sums the per-block partials of entry k; the loads of
             // different entries are in flight together
             for (int k = warp; k < K; k += nw) {
-                // up to 8 partials per lane per round, all loads issued before
-                // the adds (one L2 round trip per 256 blocks)
-                const double *Pk = P + (size_t)k * nblocks;
-                double u = 0.0;
-                for (int b0 = 0; b0 < nblocks; b0 += 256) {
-                    double w[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int b = b0 + lane + 32 * j;
-                        w[j] = b < nblocks ? __ldcg(Pk + b) : 0.0;
-                    }
-                    u += ((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7]));
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+                const double u = sum_partials(P + (size_t)k * nblocks, nblocks);
                 if (lane == 0) sm->bcast[k] = u;
             }
         } else {
@@ -328,6 +346,15 @@ struct GridTeam {
     }
 };
 
+template <class Team>
+struct IsGridTeam {
+    static constexpr bool value = false;
+};
+template <>
+struct IsGridTeam<GridTeam> {
+    static constexpr bool value = true;
+};
+
 constexpr int kMaxCluster = 16;
 
 // The CTAs of one thread-block cluster (all co-scheduled by the hardware).
@@ -359,7 +386,7 @@ struct ClusterTeam {
         slot ^= 1;
         double *buf = xch + (size_t)slot * kMaxCluster * kMaxRed;
         if (warp == 0) {
-            warp0_sum_warps<K>(*sm);
+            warp0_sum_warps<K>(*sm, nw);
             __syncwarp();
             for (int q = lane; q < (int)size * K; q += 32) {
                 const unsigned r = (unsigned)(q / K);
@@ -390,6 +417,11 @@ struct ClusterTeam {
 // takes slices s0 + w, s0 + w + nwarps, ...; lane l takes row 32 s + l.
 struct Rows {
     int64_t s0, s1, n;
+    // warps (of nw) that own at least one slice; at least 1
+    __device__ __forceinline__ int active_warps(int nw) const {
+        const int64_t k = s1 - s0;
+        return k < 1 ? 1 : k < nw ? (int)k : nw;
+    }
     template <class F>
     __device__ __forceinline__ void each(F &&f) const {
         const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
