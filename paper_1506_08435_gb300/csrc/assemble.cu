@@ -209,13 +209,25 @@ __device__ __forceinline__ int tri_index(int a, int b, int nv) {  // a <= b, pac
     return a * nv - (a * (a - 1)) / 2 + (b - a);
 }
 
+// a / b, correctly rounded, from y = the correctly rounded 1 / b: one Newton
+// correction of the quotient by the exact remainder (P. Markstein, IBM J. Res.
+// Develop. 34, 1990).  Three operations, where a division is eight to ten; for
+// several quotients by one b.  b's magnitude is kept away from the ends of the
+// range by the callers.
+__device__ __forceinline__ double quotient(double a, double b, double y) {
+    const double q = __dmul_rn(a, y);
+    return fma(fma(-b, q, a), y, q);
+}
+
 // K_e (packed upper triangle, nv(nv+1)/2 values) and |e| of every element.
-// Bound by the FP64 pipe (a warp instruction holds a sub-core for 64 cycles, a
-// division is eight to ten of them), so the operations are few: one division
-// per element (by det, nine before), 1 / |v| and |v| from one reciprocal
-// square root, the rows of vertex 0 from the zero row sums, and for a cell
-// velocity K_ab = |e| (iso G_a.G_b + lon (v.G_a)(v.G_b)) without forming D_e.
-// 90 x 101 x 84 hexahedra, 4.6M tetrahedra: 2.62 -> 1.06 ms, the pipe 84% busy.
+// Bound by the FP64 pipe (a warp instruction holds a sub-core for 64 cycles),
+// so the operations are few, though every value is the same to the last bit as
+// from plain divisions: the nine quotients by det and |e| come from one
+// reciprocal, and the minors of D_e are formed only where they could be small.
+// 90 x 101 x 84 hexahedra, 4.6M tetrahedra: 2.62 -> 1.61 ms.  (1.06 ms with
+// K_ab = |e| (iso G_a.G_b + lon (v.G_a)(v.G_b)), whose last bits differ: they
+// send a solve of thousands of CG iterations down another path, and served
+// solutions, known to 1e-9, would move by as much.)
 template <int DIM>
 __global__ void __launch_bounds__(TPB) k_element(int64_t E, const double *__restrict__ coords,
                                                  const int32_t *__restrict__ conn, int kind,
@@ -259,14 +271,30 @@ __global__ void __launch_bounds__(TPB) k_element(int64_t E, const double *__rest
         set_status(st, NN_ERR_DEGENERATE);
         return;
     }
-    const double ri = 1.0 / det;
-    const double v = fabs(det) * (DIM == 2 ? 0.5 : 1.0 / 6.0);
-    double G[DIM][DIM];
+    double v;
+    double G[DIM + 1][DIM];   // gradients of the barycentric coordinates
+    if (fabs(det) > 1e-180 && fabs(det) < 1e180) {
+        const double y = 1.0 / det;
+        v = DIM == 2 ? fabs(det) * 0.5 : quotient(fabs(det), 6.0, 1.0 / 6.0);
 #pragma unroll
-    for (int k = 0; k < DIM; ++k)
+        for (int k = 0; k < DIM; ++k)
 #pragma unroll
-        for (int p = 0; p < DIM; ++p) G[k][p] = c[k][p] * ri;
-    double K[DIM][DIM];   // rows and columns of the vertices 1 .. DIM, a <= b
+            for (int p = 0; p < DIM; ++p) G[k + 1][p] = quotient(c[k][p], det, y);
+    } else {
+        v = fabs(det) / (DIM == 2 ? 2.0 : 6.0);
+#pragma unroll
+        for (int k = 0; k < DIM; ++k)
+#pragma unroll
+            for (int p = 0; p < DIM; ++p) G[k + 1][p] = c[k][p] / det;
+    }
+#pragma unroll
+    for (int p = 0; p < DIM; ++p) {
+        double x = 0.0;
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) x += G[k + 1][p];
+        G[0][p] = -x;
+    }
+    double D[DIM][DIM];
     // symmetric positive definite: leading principal minors > 0
     auto spd = [](const double (&D)[DIM][DIM]) {
         const double d1 = D[0][0], d2 = D[0][0] * D[1][1] - D[0][1] * D[1][0];
@@ -282,7 +310,7 @@ __global__ void __launch_bounds__(TPB) k_element(int64_t E, const double *__rest
     };
     if (kind == NN_COEF_TENSOR) {
         constexpr int nc = DIM == 2 ? 3 : 6;
-        double t[nc], D[DIM][DIM];
+        double t[nc];
         bool fin = true;
 #pragma unroll
         for (int q = 0; q < nc; ++q) {
@@ -302,24 +330,6 @@ __global__ void __launch_bounds__(TPB) k_element(int64_t E, const double *__rest
             set_status(st, NN_ERR_NOT_SPD);
             return;
         }
-#pragma unroll
-        for (int b = 0; b < DIM; ++b) {
-            double DG[DIM];
-#pragma unroll
-            for (int p = 0; p < DIM; ++p) {
-                double x = 0.0;
-#pragma unroll
-                for (int r = 0; r < DIM; ++r) x += D[p][r] * G[b][r];
-                DG[p] = x * v;
-            }
-#pragma unroll
-            for (int a = 0; a <= b; ++a) {
-                double x = 0.0;
-#pragma unroll
-                for (int p = 0; p < DIM; ++p) x += G[a][p] * DG[p];
-                K[a][b] = x;
-            }
-        }
     } else {
         double vv[DIM], n2 = 0.0;
         bool fin = true;
@@ -327,73 +337,49 @@ __global__ void __launch_bounds__(TPB) k_element(int64_t E, const double *__rest
         for (int p = 0; p < DIM; ++p) {
             vv[p] = coef[e * DIM + p];
             fin = fin && isfinite(vv[p]);
-            n2 += vv[p] * vv[p];
+            n2 = fma(vv[p], vv[p], n2);
         }
         if (!fin) {
             set_status(st, NN_ERR_NUMERIC);
             return;
         }
-        const double dl = aL - aT;
-        double vn, lon;
-        if (n2 > 1e-290 && n2 < 1e290) {
-            const double rs = rsqrt(n2);
-            vn = n2 * rs;
-            lon = dl * rs;
-        } else {           // |v| = 0, or a square that may have left the range of the reciprocal root
-            vn = sqrt(n2);
-            lon = vn > 0.0 ? dl / vn : 0.0;
-        }
-        const double iso = aT * vn + DM, along = lon * n2;
+        const double vn = sqrt(n2);
+        const double iso = aT * vn + DM;
+        const double lon = vn > 0.0 ? (aL - aT) / vn : 0.0;
+#pragma unroll
+        for (int p = 0; p < DIM; ++p)
+#pragma unroll
+            for (int r = 0; r < DIM; ++r) D[p][r] = lon * vv[p] * vv[r] + (p == r ? iso : 0.0);
         // D_e = iso I + lon v v': with lon >= 0 and iso not tiny beside lon |v|^2
         // its minors are positive by a wide margin (d2 >= (iso / trace) D00 D11,
         // d3 >= (iso / trace)^2 D00 D11 D22); otherwise they are formed
-        if (!(dl >= 0.0 && iso > 1e-5 * along && iso > 1e-90 && along < 1e90 && iso < 1e90)) {
-            double D[DIM][DIM];
-#pragma unroll
-            for (int p = 0; p < DIM; ++p)
-#pragma unroll
-                for (int r = 0; r < DIM; ++r) D[p][r] = lon * vv[p] * vv[r] + (p == r ? iso : 0.0);
-            if (!spd(D)) {
-                set_status(st, NN_ERR_NOT_SPD);
-                return;
-            }
+        const double along = lon * n2;
+        if (!(aL >= aT && iso > 1e-5 * along && iso > 1e-90 && along < 1e90 && iso < 1e90) && !spd(D)) {
+            set_status(st, NN_ERR_NOT_SPD);
+            return;
         }
-        double vg[DIM];
+    }
+    // DG[b][p] = sum_q D[p][q] G[b][q]
+    double DG[nv][DIM];
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) {
+    for (int b = 0; b < nv; ++b)
+#pragma unroll
+        for (int p = 0; p < DIM; ++p) {
             double x = 0.0;
 #pragma unroll
-            for (int p = 0; p < DIM; ++p) x += vv[p] * G[a][p];
-            vg[a] = x;
+            for (int q = 0; q < DIM; ++q) x = fma(D[p][q], G[b][q], x);
+            DG[b][p] = x;
         }
-        const double vi = v * iso, vl = v * lon;
-#pragma unroll
-        for (int b = 0; b < DIM; ++b) {
-            const double wb = vl * vg[b];
-#pragma unroll
-            for (int a = 0; a <= b; ++a) {
-                double x = 0.0;
-#pragma unroll
-                for (int p = 0; p < DIM; ++p) x += G[a][p] * G[b][p];
-                K[a][b] = vi * x + vg[a] * wb;
-            }
-        }
-    }
     double *out = Ke + e * nk;
-    double k00 = 0.0;
 #pragma unroll
-    for (int b = 0; b < DIM; ++b) {
-        double x = 0.0;
+    for (int a = 0; a < nv; ++a)
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) x += a <= b ? K[a][b] : K[b][a];
-        out[1 + b] = -x;
-        k00 += x;
-    }
-    out[0] = k00;
+        for (int b = a; b < nv; ++b) {
+            double x = 0.0;
 #pragma unroll
-    for (int a = 0; a < DIM; ++a)
-#pragma unroll
-        for (int b = a; b < DIM; ++b) out[tri_index(a + 1, b + 1, nv)] = K[a][b];
+            for (int p = 0; p < DIM; ++p) x = fma(G[a][p], DG[b][p], x);
+            out[tri_index(a, b, nv)] = v * x;
+        }
     vol[e] = v;
 }
 
@@ -403,8 +389,9 @@ __global__ void __launch_bounds__(TPB) k_element(int64_t E, const double *__rest
 // != 0 its row-sum lumping |e| delta_ab/(d+1).  Of a node's eight lanes, lane
 // b < nv adds vertex b's entry of K, lane 4 + b that of M (an element's
 // vertices differ, so no two lanes meet); eight incidences are fetched ahead of
-// their additions.  Bound by L1 (82%: the shared-memory sums); 0.87 ms at the
-// size above, where columns and sums took 0.69 + 1.20 ms.
+// their additions.  Bound by L1 (82%: the shared-memory sums); 0.75 ms at the
+// size above, where columns and sums took 0.69 + 1.20 ms.  Every sum is rounded
+// as one multiply-add per term in that order.
 template <int nv>
 __global__ void __launch_bounds__(kNodeBlock) k_node_rows(int64_t N, const int32_t *__restrict__ conn,
                                                           const int64_t *__restrict__ iptr,
@@ -466,23 +453,28 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_rows(int64_t N, const int32
     for (int o = 16; o >= kNodeLanes; o >>= 1) mw = max(mw, __shfl_xor_sync(0xffffffffu, mw, o));
     constexpr int U = 8;
     for (int k0 = 0; k0 < mw; k0 += U) {
-        double x[U];
+        double x[U], y[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             x[u] = 0.0;
+            y[u] = 1.0;
             if (k0 + u < m) {
                 const int code = list[g][k0 + u], e = code / nv, a = code - e * nv;
                 if (half == 0) {
                     if (mine) x[u] = Ke[(int64_t)e * nk + tri_index(a < b ? a : b, a < b ? b : a, nv)];
                 } else if (mine) {
-                    x[u] = vol[e] * (a == b ? md : mo);
+                    x[u] = vol[e];
+                    y[u] = a == b ? md : mo;
                 }
-                if (f_elem && l == 0) fr += f_elem[e] * vol[e];
+                if (f_elem && l == 0) fr += quotient(__dmul_rn(f_elem[e], vol[e]), nv, 1.0 / nv);
             }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (mine && k0 + u < m) sum[at[g][(k0 + u) * nv + b]] += x[u];
+            if (mine && k0 + u < m) {
+                double &t = sum[at[g][(k0 + u) * nv + b]];
+                t = fma(x[u], y[u], t);
+            }
             __syncwarp();
         }
     }
@@ -490,7 +482,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_rows(int64_t N, const int32
         Kval[r0 + k] = acc[k];
         if (Mval) Mval[r0 + k] = acc[kMaxRow + k];
     }
-    if (in && l == 0) F[r] = f_elem ? fr / nv : 0.0;
+    if (in && l == 0) F[r] = fr;
 }
 
 // ------------------------------------------------------------------ elimination

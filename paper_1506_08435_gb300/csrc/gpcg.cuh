@@ -372,7 +372,18 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
         for (;;) {
             if (can_reside && C.res_warps > 0) {
                 if constexpr (can_reside) {
-                    const int e = cg_resident(T, R, A, B, v, C, st, ftol2, C.res_warps);
+                    // (copies for the call: what is passed by reference lives in the
+                    // stack frame, and the passes here would reload it at every use)
+                    GridTeam t = T;
+                    GpcgStats s = st;
+                    const Rows r = R;
+                    const Op a = A;
+                    const Bounds<V> b = B;
+                    const GpcgVecs<V> w = v;
+                    const GpcgCtl c = C;
+                    const int e = cg_resident(t, r, a, b, w, c, s, ftol2, c.res_warps);
+                    T = t;
+                    st = s;
                     if (e == ST_TIMEOUT) return ST_TIMEOUT;
                     if (e != 0) break;
                 }

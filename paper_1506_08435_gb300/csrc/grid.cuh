@@ -157,7 +157,10 @@ __device__ bool step_outputs(Team &T, const Rows &R, const GridArgs &a, const do
 // (mid-size systems, whose slices per block fit in shared memory);
 // 3 (mixed modes) = the FP32 operator of the inner products streamed through
 // shared memory by bulk asynchronous copies, D slices in flight per warp
-// (operators far larger than L2).
+// (operators far larger than L2);
+// 4, 5 = the operator as with 2 and 0, and the pipelined CG phase with its
+// vectors in shared memory (cg_resident.cuh; kernels of their own, as its code
+// costs the plain phase registers).
 template <int FMT, int MODE, int CGV, int TPB>
 __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k_solve_grid(GridArgs a) {
     __shared__ RedSmem sm;
@@ -169,8 +172,9 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k
     double *x = a.v64[0];
     R.each([&](int64_t i) { x[i] = a.c_in[a.free_node[i]]; });
     // shared memory of the resident CG phase (behind the operator of FMT 2)
-    constexpr bool RES = CGV == 2 && TPB == 512 && (FMT == 2 || FMT == 0);
-    unsigned char *res = op_smem + a.res_offset;
+    constexpr bool RES = FMT == 4 || FMT == 5, LOCAL = FMT == 2 || FMT == 4;
+    static_assert(!RES || (CGV == 2 && TPB == 512), "the resident CG phase is form 2 in 512-thread blocks");
+    [[maybe_unused]] unsigned char *res = op_smem + a.res_offset;
     SellF64Local Aloc{};
     SellF32DiffLocal A32loc{};
     SellF32DiffTma A32tma{};
@@ -187,7 +191,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k
         A32tma.error = &a.bar->error;
         A32tma.setup(op_smem);
     }
-    if constexpr (FMT == 2) {
+    if constexpr (LOCAL) {
         // stage entries [e0, e1) of this block's slices: columns, then values
         constexpr bool MIX = mode_mixed(MODE);
         const int64_t e0 = a.A.sptr[R.s0], e1 = a.A.sptr[R.s1];
@@ -230,7 +234,14 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k
                 v.res = reinterpret_cast<float *>(res + a.res_table);
             }
             MixedStats ms;
-            if constexpr (FMT == 2)
+            if constexpr (RES) {
+                SellF32DiffResX<LOCAL> A32r;
+                if constexpr (LOCAL) static_cast<SellF32DiffLocal &>(A32r) = A32loc;
+                else static_cast<SellF32Diff &>(A32r) = a.A32;
+                status = mixed_solve<CGV, inner_cg_form(MODE, CGV), true>(T, R, a.A, A32r, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
+                                                 a.v32[11], v64, a.rtol * den, a.inner_rtol, a.max_ref,
+                                                 a.ctl.max_spmv, a.inner_cap, a.ctl, a.ctl, ms);
+            } else if constexpr (LOCAL)
                 status = mixed_solve<CGV, inner_cg_form(MODE, CGV), true>(T, R, a.A, A32loc, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
                                                  a.v32[11], v64, a.rtol * den, a.inner_rtol, a.max_ref,
                                                  a.ctl.max_spmv, a.inner_cap, a.ctl, a.ctl, ms);
@@ -238,13 +249,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k
                 status = mixed_solve<CGV, inner_cg_form(MODE, CGV), (TPB < 512)>(T, R, a.A, A32tma, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
                                                  a.v32[11], v64, a.rtol * den, a.inner_rtol, a.max_ref,
                                                  a.ctl.max_spmv, a.inner_cap, a.ctl, a.ctl, ms);
-            else if constexpr (RES) {
-                SellF32DiffRes A32r;
-                static_cast<SellF32Diff &>(A32r) = a.A32;
-                status = mixed_solve<CGV, inner_cg_form(MODE, CGV), true>(T, R, a.A, A32r, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
-                                                 a.v32[11], v64, a.rtol * den, a.inner_rtol, a.max_ref,
-                                                 a.ctl.max_spmv, a.inner_cap, a.ctl, a.ctl, ms);
-            } else
+            else
                 status = mixed_solve<CGV, inner_cg_form(MODE, CGV), true>(T, R, a.A, a.A32, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
                                                  a.v32[11], v64, a.rtol * den, a.inner_rtol, a.max_ref,
                                                  a.ctl.max_spmv, a.inner_cap, a.ctl, a.ctl, ms);
@@ -274,13 +279,14 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k
             c.face_tol = 0.5 * c.tol;
             GpcgStats gs;
             const Bounds<double> B{a.lo, a.hi, nullptr, nullptr};
-            if constexpr (FMT == 0 && RES) {
-                SellF64Res Ar;
-                static_cast<SellF64 &>(Ar) = a.A;
-                status = gpcg_solve<GridTeam, SellF64Res, double, CGV>(T, R, Ar, B, v, c, gs);
+            if constexpr (RES) {
+                SellF64ResX<LOCAL> Ar;
+                if constexpr (LOCAL) static_cast<SellF64Local &>(Ar) = Aloc;
+                else static_cast<SellF64 &>(Ar) = a.A;
+                status = gpcg_solve<GridTeam, SellF64ResX<LOCAL>, double, CGV>(T, R, Ar, B, v, c, gs);
             } else if constexpr (FMT == 0)
                 status = gpcg_solve<GridTeam, SellF64, double, CGV>(T, R, a.A, B, v, c, gs);
-            else if constexpr (FMT == 2)
+            else if constexpr (LOCAL)
                 status = gpcg_solve<GridTeam, SellF64Local, double, CGV>(T, R, Aloc, B, v, c, gs);
             else
                 status = gpcg_solve<GridTeam, CsrF64, double, CGV>(T, R, a.Acsr, B, v, c, gs);
@@ -310,9 +316,12 @@ using GridKernel = void (*)(GridArgs);
 // FP32 SELL operator streamed through shared memory by bulk copies.
 constexpr int FMT_SELL_SMEM = 2;
 constexpr int FMT_SELL_TMA = 3;
+// ... and the first two with the resident CG phase.
+constexpr int FMT_SELL_SMEM_RES = 4;
+constexpr int FMT_SELL_RES = 5;
 
 // Kernel of one mode for format fmt (NN_FMT_SELL / NN_FMT_CSR /
-// FMT_SELL_SMEM), CG variant cgv (0, 1, 2; 3 = textbook CG with the SSOR
+// FMT_SELL_SMEM ...), CG variant cgv (0, 1, 2; 3 = textbook CG with the SSOR
 // preconditioner, FP64 modes) and threads per block tpb (256, 512, 768);
 // nullptr if that combination is not built.
 GridKernel grid_kernel_steady(int fmt, int cgv, int tpb);

@@ -396,31 +396,25 @@ struct SellF32DiffTma {
     }
 };
 
-// The operators of kernels whose CG phase keeps its vectors in shared memory
-// (cg_resident.cuh): in shared memory themselves, or, as these two, read from
-// global memory (the same entries in the same order: the results are the same
-// bits).
-struct SellF64Res : SellF64X<false> {};
-struct SellF32DiffRes : SellF32DiffX<false> {};
+// The same operators by another type, for the kernels whose CG phase keeps its
+// vectors in shared memory (cg_resident.cuh): in shared memory themselves or
+// read from global memory (the same entries in the same order: the results are
+// the same bits).
+template <bool LOCAL>
+struct SellF64ResX : SellF64X<LOCAL> {};
+template <bool LOCAL>
+struct SellF32DiffResX : SellF32DiffX<LOCAL> {};
 template <class Op>
 struct IsResidentOp {
     static constexpr bool value = false;
 };
-template <>
-struct IsResidentOp<SellF64X<true>> {
-    static constexpr bool value = true, local = true;
+template <bool L>
+struct IsResidentOp<SellF64ResX<L>> {
+    static constexpr bool value = true, local = L;
 };
-template <>
-struct IsResidentOp<SellF32DiffX<true>> {
-    static constexpr bool value = true, local = true;
-};
-template <>
-struct IsResidentOp<SellF64Res> {
-    static constexpr bool value = true, local = false;
-};
-template <>
-struct IsResidentOp<SellF32DiffRes> {
-    static constexpr bool value = true, local = false;
+template <bool L>
+struct IsResidentOp<SellF32DiffResX<L>> {
+    static constexpr bool value = true, local = L;
 };
 
 // Whether an operator streams through L2 (large systems): the vector passes
@@ -429,8 +423,10 @@ template <bool L>
 __device__ __forceinline__ bool op_streams(const SellF64X<L> &A) { return A.stream; }
 template <bool L>
 __device__ __forceinline__ bool op_streams(const SellF32DiffX<L> &A) { return A.stream; }
-__device__ __forceinline__ bool op_streams(const SellF64Res &A) { return A.stream; }
-__device__ __forceinline__ bool op_streams(const SellF32DiffRes &A) { return A.stream; }
+template <bool L>
+__device__ __forceinline__ bool op_streams(const SellF64ResX<L> &A) { return A.stream; }
+template <bool L>
+__device__ __forceinline__ bool op_streams(const SellF32DiffResX<L> &A) { return A.stream; }
 __device__ __forceinline__ bool op_streams(const SellF32DiffTma &) { return true; }
 template <class Op>
 __device__ __forceinline__ bool op_streams(const Op &) { return false; }

@@ -452,9 +452,11 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     // (cg_resident.cuh) in 512-thread blocks, which the smallest systems gain
     // from as well (50 x 50: 5.3 ms in 19 blocks of 256 threads, 3.9 ms here);
     // their slices are spread one to a block as far as there are SMs (12 to 76
-    // blocks measure alike there).
+    // blocks measure alike there).  Served solves (force_tpb) do without: blocks
+    // of several requests share an SM, which its shared memory would not allow,
+    // and what a request returns stays the same bits.
     const bool mid = !driver && !large && slices <= (int64_t)4 * 8 * sms;
-    const bool on_chip = mid && fmt == NN_FMT_SELL && a.ctl.cg_variant == 2 && mode != MODE_MIXED;
+    const bool on_chip = mid && force_tpb == 0 && fmt == NN_FMT_SELL && a.ctl.cg_variant == 2 && mode != MODE_MIXED;
     if (mid && (on_chip || slices > (int64_t)8 * sms / 2)) tpb = 512;
     if (!driver && (force_tpb == 256 || force_tpb == 512)) tpb = force_tpb;
     if (large && (a.ctl.cg_variant == 0 || a.ctl.cg_variant == 3) && fmt == NN_FMT_SELL && force_tpb != 512)
@@ -520,14 +522,15 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
         const size_t op = (size_t)most * (4 + vbytes), table = ((size_t)(deep + 1) * 4 + 15) / 16 * 16;
         const size_t vecs = table + (size_t)kResVectors * deep * 32 * vbytes;
         const char *rw = getenv("NNQP_RES_WARPS");
-        const bool form = a.ctl.cg_variant == 2 && !a.ctl.cg_bound_stop && mode != MODE_MIXED && !(rw && atoi(rw) < 1);
+        const bool form = on_chip && !a.ctl.cg_bound_stop && !(rw && atoi(rw) < 1);
         const bool both = form && op + vecs <= kSmemBytes;
         // (the resident phase is the same with either operator: whether it is
         // taken does not depend on NNQP_SMEM_OP)
         const bool resident = both || (form && op > kSmemOperatorBytes && vecs <= kSmemBytes);
         const bool local = smem_op && op > 0 && (resident ? both : op <= kSmemOperatorBytes);
         const size_t bytes = (local ? op : 0) + (resident ? vecs : 0);
-        GridKernel ks = bytes ? grid_kernel(mode, local ? FMT_SELL_SMEM : NN_FMT_SELL, a.ctl.cg_variant, tpb) : nullptr;
+        const int f = resident ? (local ? FMT_SELL_SMEM_RES : FMT_SELL_RES) : FMT_SELL_SMEM;
+        GridKernel ks = bytes ? grid_kernel(mode, f, a.ctl.cg_variant, tpb) : nullptr;
         // the attribute is set to the same budget by every caller (solves on
         // other host threads may launch this kernel at the same time)
         if (ks && cudaFuncSetAttribute((const void *)ks, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -4,6 +4,10 @@
 namespace nnqp {
 
 GridKernel grid_kernel_steady(int fmt, int cgv, int tpb) {
+    if (fmt == FMT_SELL_SMEM_RES || fmt == FMT_SELL_RES) {
+        if (tpb != 512 || cgv != 2) return nullptr;
+        return fmt == FMT_SELL_RES ? k_solve_grid<5, MODE_STEADY, 2, 512> : k_solve_grid<4, MODE_STEADY, 2, 512>;
+    }
     if (fmt == FMT_SELL_SMEM) {
         if (tpb != 512) return nullptr;
         switch (cgv) {

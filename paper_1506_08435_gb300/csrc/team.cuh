@@ -153,12 +153,13 @@ __device__ __forceinline__ void warp_stage(const double (&v)[K], RedSmem &sm) {
 }
 
 // Cross-warp stage: the per-warp totals sm.warp[w][k] (w < nw) are summed by
-// the calling warp and stored to sm.bcast[k].  An FP64 warp instruction takes
-// 64 cycles of its sub-core whatever its active lanes (measured), an addition
-// behind a shuffle 118, so the lanes are packed for few dependent additions: L
-// lanes per entry, each adding every L-th warp's total, then log2 L shuffles
-// (16 warps: K <= 4 one addition and three shuffles for all entries, K <= 8
-// three and two; packing 32 / nw entries per instruction took 8 and 12).
+// the calling warp in butterfly order and stored to sm.bcast[k].  An FP64 warp
+// instruction takes 64 cycles of its sub-core whatever its active lanes
+// (measured), an addition behind a shuffle 118, so the lanes are packed for few
+// dependent additions: L lanes per entry, each adding the totals w, w + L, ...
+// of the butterfly's outer levels itself, then log2 L shuffles (16 warps: K <= 4
+// one addition and three shuffles for all entries, K <= 8 two and two; packing
+// 32 / nw entries per instruction took 8 and 12 behind shuffles).
 template <int K>
 __device__ __forceinline__ void warp0_sum_warps(RedSmem &sm, int nw) {
     constexpr int P = K <= 4 ? 4 : K <= 8 ? 8 : K <= 16 ? 16 : 32;
@@ -166,8 +167,25 @@ __device__ __forceinline__ void warp0_sum_warps(RedSmem &sm, int nw) {
     const int lane = threadIdx.x & 31, j = lane % L;
     for (int k0 = 0; k0 < K; k0 += P) {
         const int k = k0 + lane / L;
-        double t = (k < K && j < nw) ? sm.warp[j][k] : 0.0;
-        for (int w = j + L; w < nw; w += L) t += k < K ? sm.warp[w][k] : 0.0;
+        double t;
+        if constexpr (L >= 4) {
+            // kMaxWarps / L terms, halved level by level (absent warps add 0)
+            constexpr int M = kMaxWarps / L;
+            double w[M];
+#pragma unroll
+            for (int i = 0; i < M; ++i) w[i] = (k < K && j + i * L < nw) ? sm.warp[j + i * L][k] : 0.0;
+            if (nw > 16)
+#pragma unroll
+                for (int i = 0; i < M / 2; ++i) w[i] += w[i + M / 2];
+            if (nw > 8)
+#pragma unroll
+                for (int i = 0; i < M / 4; ++i) w[i] += w[i + M / 4];
+            if (M >= 8 && nw > 4) w[0] += w[M / 8];
+            t = w[0];
+        } else {
+            t = (k < K && j < nw) ? sm.warp[j][k] : 0.0;
+            for (int w = j + L; w < nw; w += L) t += k < K ? sm.warp[w][k] : 0.0;
+        }
 #pragma unroll
         for (int o = L >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (j == 0 && k < K) sm.bcast[k] = t;
