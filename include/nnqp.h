@@ -433,20 +433,23 @@ nn_status nn_shard_spmv(int64_t nrows, const int64_t *local_rowptr, const int32_
 
 /* --------------------------------------------------------------- batching */
 
-/* Solves `count` independent steady systems in ONE persistent launch.
+/* Solves `count` independent steady systems in one persistent launch (or one
+ * per cluster size).
  * Each system is solved either by one thread block, or by one thread-block
- * cluster of 4/8/16 CTAs on as many SMs (hardware cluster barriers,
- * reductions through distributed shared memory); systems are taken largest
- * first from a device work counter.  The shape is the autotuner's choice
- * (nn_batch_autotune) or 256 threads x 1 CTA.  c[i] is the full node vector
+ * cluster on as many SMs (hardware cluster barriers, reductions through
+ * distributed shared memory); systems are taken largest first from a device
+ * work counter.  The shape is the autotuner's choice (nn_batch_autotune) or
+ * 512 threads x up to 16 CTAs: each system gets a cluster of 1/2/4/8/16 CTAs by
+ * its size, one launch per cluster size side by side.  c[i] is the full node vector
  * of system i (device memory).  infos: NULL or [count].  Mixed precision
  * uses FP32 inner solves with FP64 refinement per system.  Synchronizes. */
 nn_status nn_batch_solve(int count, nn_system *const *systems, double *const *c, const nn_solve_opts *o,
                          void *stream, nn_solve_info *infos);
 
 /* Times candidate launch shapes (threads per block x CTAs per system:
- * 256x4, 256x8, 256x16; for batches whose largest system has at most 8192
- * free unknowns 256x1, 512x1, 256x4, 256x8) on the whole batch solved to the
+ * 512x16 (up to 16 CTAs, by size), 512x8, 256x8, 256x16; for batches whose
+ * largest system has at most 8192 free unknowns 512x16, 256x1, 512x1, 256x4,
+ * 256x8) on the whole batch solved to the
  * requested tolerance, and keeps the fastest for later nn_batch_solve calls
  * in this process.  *best_shape receives threads * 100 + CTAs (e.g. 25608). */
 nn_status nn_batch_autotune(int count, nn_system *const *systems, const nn_solve_opts *o, void *stream,

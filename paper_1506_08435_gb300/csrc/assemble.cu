@@ -553,7 +553,8 @@ __global__ void k_red_fill(int64_t NF, const int32_t *free_node, const int32_t *
     offcnt[i] = (o - arow[i]) - 1;
 }
 
-__global__ void k_slice_width(int64_t NF, int64_t nslices, const int64_t *offcnt, int64_t *wslots) {
+__global__ void k_slice_width(int64_t NF, int64_t nslices, const int64_t *offcnt, int64_t *wslots,
+                              unsigned long long *widest) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= nslices) return;
     int64_t w = 0;
@@ -562,6 +563,7 @@ __global__ void k_slice_width(int64_t NF, int64_t nslices, const int64_t *offcnt
         if (i < NF && offcnt[i] > w) w = offcnt[i];
     }
     wslots[s] = 32 * (w + (w & 1));   // even width: entries are stored in pairs
+    if (widest) atomicMax(widest, (unsigned long long)wslots[s]);
 }
 
 // One thread per slot row: writes the row's off-diagonals into its SELL
@@ -880,7 +882,12 @@ nn_status assemble_impl(const nn_problem *p, const nn_assemble_opts *o, cudaStre
     TRYF(T.a.alloc(&wslots, nslices, st));
     int64_t *sptr;
     TRYF(s->arena.alloc(&sptr, nslices + 1, st));
-    (k_slice_width<<<nblk(nslices), TPB, 0, st>>>(NF, nslices, offcnt, wslots), ::nnqp::count_launch());
+    // two norms and the widest slice, read back together at the end
+    double *dn;
+    TRYF(T.a.alloc(&dn, 3 + 1024, st));
+    CUF(cudaMemsetAsync(dn, 0, 3 * sizeof(double), st));
+    (k_slice_width<<<nblk(nslices), TPB, 0, st>>>(NF, nslices, offcnt, wslots,
+                                                  reinterpret_cast<unsigned long long *>(dn + 2)), ::nnqp::count_launch());
     int64_t *scratch3;
     TRYF(T.a.alloc(&scratch3, scan_tmp_elems(nslices + 1) + 64, st));
     CUF(exclusive_scan(wslots, sptr, nslices, scratch3, st));
@@ -917,13 +924,12 @@ nn_status assemble_impl(const nn_problem *p, const nn_assemble_opts *o, cudaStre
                                                      transient ? s->M64.val : nullptr, s->rsum32, s->dinv32,
                                                      s->dinv64, s->diag64), ::nnqp::count_launch());
     // ---- norms
-    double *dn;
-    TRYF(T.a.alloc(&dn, 2 + 1024, st));
-    CUF(det_max(rabs, NF, dn, dn + 2, st));
-    CUF(det_sumsq(s->b0, NF, dn + 1, dn + 2, st));
-    double hn[2];
-    CUF(cudaMemcpyAsync(hn, dn, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CUF(det_max(rabs, NF, dn, dn + 3, st));
+    CUF(det_sumsq(s->b0, NF, dn + 1, dn + 3, st));
+    double hn[3];
+    CUF(cudaMemcpyAsync(hn, dn, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
     CUF(cudaStreamSynchronize(st));
+    std::memcpy(&s->max_slice_slots, &hn[2], sizeof(int64_t));
     s->anorm_inf = hn[0];
     s->b0norm = std::sqrt(hn[1]);
     s->has_csr = true;  // the reduced CSR is always kept (small next to SELL; used by nn_spmv)

@@ -19,12 +19,45 @@ BatchKernel pick_kernel(bool mixed, int tpb, int cluster, int cgv) {
     return mixed ? batch_kernel_mixed(tpb, cluster, cgv) : batch_kernel_fp64(tpb, cluster, cgv);
 }
 
-// Launch shape of the batch kernel: threads per block and CTAs per
-// instance (1 = one block per instance, > 1 = a cluster per instance).
+// Launch shape of the batch kernel: threads per block and CTAs per instance
+// (1 = one block per instance, > 1 = a cluster per instance).  512 threads with
+// more than one CTA is the resident kernel with at most that many CTAs per
+// instance: each instance gets a cluster of its own size (res_cluster).
+//
+// The default is 512 x 16.  A batch of 40 instances of 20 x 20 to 120 x 120
+// cells in FP64: one 256-thread block per instance (the former default) 590 ms,
+// bounded by the largest instance on one SM; clusters of 16 x 256 threads with
+// form 0 / 2 of CG 105 / 104 ms; this 61 ms.
 struct BatchShape {
-    int tpb = 256;
-    int cluster = 1;
+    int tpb = 512;
+    int cluster = 16;
 };
+bool resident_shape(const BatchShape &s) { return s.tpb == 512 && s.cluster > 1; }
+
+// Dynamic shared memory a CTA of the resident kernel may take (its static 22 KB
+// come on top).
+constexpr size_t kBatchSmemBytes = 204 * 1024;
+
+// Where an instance of the resident kernel runs: CTAs of its cluster (0 = it
+// does not fit: the 256-thread cluster kernel takes it) and whether its operator
+// is in shared memory.  As few CTAs as give each at most `target` slices -- an
+// iteration's barrier and sums cost the same for 1 and 28 slices a CTA -- and
+// more where that is what the operator needs to fit.
+struct ResPlace {
+    int cluster = 0;
+    bool local = false;
+};
+ResPlace res_cluster(const nn_system *s, int vbytes, int64_t target, int most) {
+    const int64_t slices = s->A64.nslices;
+    for (int c = 1; c <= most; c *= 2) {
+        const int64_t per = (slices + c - 1) / c;
+        if (per <= target && batch_res_bytes(per, s->max_slice_slots, vbytes) <= kBatchSmemBytes) return {c, true};
+    }
+    const int64_t per = (slices + most - 1) / most;
+    if (batch_res_bytes(per, s->max_slice_slots, vbytes) <= kBatchSmemBytes) return {most, true};
+    if (batch_res_bytes(per, 0, vbytes) <= kBatchSmemBytes) return {most, false};
+    return {};
+}
 BatchShape g_tuned;          // process-wide choice of the autotuner
 bool g_have_tuned = false;
 
@@ -59,6 +92,8 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         set_error("nn_batch_solve runs GPCG on the SELL format");
         return NN_ERR_INVALID_ARG;
     }
+    // (the resident kernel has the pipelined CG form without the crossing count)
+    if (resident_shape(shape) && (getenv("NNQP_BATCH_CG_VARIANT") || getenv("NNQP_CG_BOUND_STOP"))) shape = {256, 1};
     std::vector<BatchInst> h(count);
     size_t w64 = 0, w32 = 0;
     for (int i = 0; i < count; ++i) {
@@ -120,11 +155,56 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
             b.w32 = nullptr;
         }
     }
-    // largest first
+    // largest first, by class of launch
     std::vector<int> order(count);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(),
                      [&](int a, int b) { return systems[a]->nnzF > systems[b]->nnzF; });
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    struct Launch {
+        BatchShape shape;
+        bool local = false;
+        int first = 0, count = 0;
+        size_t smem = 0;
+    };
+    std::vector<Launch> launches;
+    if (!resident_shape(shape)) {
+        launches.push_back({shape, false, 0, count, 0});
+    } else {
+        // slices per CTA: what spreads the whole batch over the SMs, from 4 (a
+        // warp each) to 24 (three a warp).  Measured with 8 / 16 / 24 / 36: 40
+        // instances of 20 to 120 cells a side 66 / 60 / 63 / 61 ms, 20 mixed ones
+        // of 30 to 90 19.6 / 19.6 / 16.9 / 18.7 ms; 8 small ones of 20 to 50, which
+        // do not fill the device, 3.1 ms with 4 and 7.4 ms with 36.
+        int64_t total = 0;
+        for (int i = 0; i < count; ++i) total += systems[i]->A64.nslices;
+        const int64_t target = std::min<int64_t>(24, std::max<int64_t>(4, total / sms));
+        const int vbytes = mixed ? 4 : 8;
+        std::vector<ResPlace> place(count);
+        for (int i = 0; i < count; ++i) place[i] = res_cluster(systems[i], vbytes, target, shape.cluster);
+        auto key = [&](int i) { return place[i].cluster == 0 ? 64 : 2 * place[i].cluster + (place[i].local ? 0 : 1); };
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key(a) > key(b); });
+        for (int q = 0; q < count; ++q) {
+            const int i = order[q];
+            const ResPlace &pl = place[i];
+            if (q == 0 || key(i) != key(order[q - 1])) {
+                Launch l;
+                l.shape = pl.cluster ? BatchShape{512, pl.cluster} : BatchShape{256, 16};
+                l.local = pl.local;
+                l.first = q;
+                launches.push_back(l);
+            }
+            Launch &l = launches.back();
+            ++l.count;
+            if (pl.cluster) {
+                const int64_t per = (systems[i]->A64.nslices + pl.cluster - 1) / pl.cluster;
+                l.smem = std::max(l.smem, batch_res_bytes(per, pl.local ? systems[i]->max_slice_slots : 0, vbytes));
+            }
+        }
+    }
+    const int nl = (int)launches.size();
     BatchInst *dinst;
     int *dorder;
     unsigned *dnext;
@@ -132,12 +212,12 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
     double *dsc;
     NN_TRY(S.a.alloc(&dinst, count, st));
     NN_TRY(S.a.alloc(&dorder, count, st));
-    NN_TRY(S.a.alloc(&dnext, 1, st));
+    NN_TRY(S.a.alloc(&dnext, nl, st));
     NN_TRY(S.a.alloc(&dcnt, (size_t)count * kBatchCounters, st));
     NN_TRY(S.a.alloc(&dsc, (size_t)2 * count, st));
     NN_CUDA_TRY(cudaMemcpyAsync(dinst, h.data(), sizeof(BatchInst) * count, cudaMemcpyHostToDevice, st));
     NN_CUDA_TRY(cudaMemcpyAsync(dorder, order.data(), sizeof(int) * count, cudaMemcpyHostToDevice, st));
-    NN_CUDA_TRY(cudaMemsetAsync(dnext, 0, sizeof(unsigned), st));
+    NN_CUDA_TRY(cudaMemsetAsync(dnext, 0, sizeof(unsigned) * nl, st));
     NN_CUDA_TRY(cudaMemsetAsync(dcnt, 0, sizeof(int64_t) * count * kBatchCounters, st));
     GpcgCtl ctl;
     ctl.tol = 0;
@@ -157,28 +237,51 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
     if (const char *e = getenv("NNQP_GP_MAX")) ctl.gp_max = atoi(e);
     if (const char *e = getenv("NNQP_ETA1")) ctl.eta1 = atof(e);
     if (const char *e = getenv("NNQP_ETA2")) ctl.eta2 = atof(e);
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int tpb = shape.cluster > 1 ? 256 : shape.tpb;
-    BatchKernel k = pick_kernel(mixed, tpb, shape.cluster, ctl.cg_variant);
-    if (!k) {
-        set_error("nn_batch_solve: no kernel for %d threads x %d CTAs, CG variant %d", tpb, shape.cluster,
-                  ctl.cg_variant);
-        return NN_ERR_INVALID_ARG;
+    // The classes run side by side: the first on the caller's stream, each other
+    // one on a stream of its own between two events of the caller's.
+    struct Side {
+        cudaStream_t st = nullptr;
+        cudaEvent_t done = nullptr;
+        ~Side() {
+            if (done) cudaEventDestroy(done);
+            if (st) cudaStreamDestroy(st);   // (its work is joined or, after an error, finishes by itself)
+        }
+    };
+    std::vector<Side> sides(std::max(nl - 1, 0));
+    struct Events {
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        ~Events() {
+            if (e0) cudaEventDestroy(e0);
+            if (e1) cudaEventDestroy(e1);
+        }
+    } ev;
+    NN_CUDA_TRY(cudaEventCreate(&ev.e0));
+    NN_CUDA_TRY(cudaEventCreate(&ev.e1));
+    for (Side &x : sides) {
+        NN_CUDA_TRY(cudaStreamCreateWithFlags(&x.st, cudaStreamNonBlocking));
+        NN_CUDA_TRY(cudaEventCreateWithFlags(&x.done, cudaEventDisableTiming));
     }
-    cudaEvent_t e0, e1;
-    NN_CUDA_TRY(cudaEventCreate(&e0));
-    NN_CUDA_TRY(cudaEventCreate(&e1));
-    if (shape.cluster <= 1) {
-        int per = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, tpb, 0);
-        const int grid = std::max(1, std::min(count, std::max(per, 1) * sms));
-        cudaEventRecord(e0, st);
-        (k<<<grid, tpb, 0, st>>>(dinst, dorder, count, dnext, ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc),
-         count_launch());
-    } else {
-        const int C = shape.cluster;
+    // one launch of class l on stream q
+    auto launch = [&](const Launch &l, unsigned *next, cudaStream_t q) -> nn_status {
+        const bool res = resident_shape(shape) && l.shape.tpb == 512;
+        const int C = l.shape.cluster, tpb = res ? kBatchResThreads : C > 1 ? 256 : l.shape.tpb;
+        BatchKernel k = res ? (mixed ? batch_res_kernel_mixed(l.local) : batch_res_kernel_fp64(l.local))
+                            : pick_kernel(mixed, tpb, C, ctl.cg_variant);
+        if (!k) {
+            set_error("nn_batch_solve: no kernel for %d threads x %d CTAs, CG variant %d", tpb, C, ctl.cg_variant);
+            return NN_ERR_INVALID_ARG;
+        }
+        if (!res && C <= 1) {
+            int per = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, tpb, 0);
+            const int grid = std::max(1, std::min(l.count, std::max(per, 1) * sms));
+            (k<<<grid, tpb, 0, q>>>(dinst, dorder + l.first, l.count, next, ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc),
+             count_launch());
+            return NN_OK;
+        }
+        if (res)
+            NN_CUDA_TRY(cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kBatchSmemBytes));
         if (C > 8) NN_CUDA_TRY(cudaFuncSetAttribute((const void *)k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
@@ -186,27 +289,44 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         attr[0].val.clusterDim.x = C;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
-        cfg.blockDim = dim3(256);
+        cfg.blockDim = dim3(tpb);
         cfg.gridDim = dim3(C * std::max(1, sms / C));
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = st;
+        cfg.dynamicSmemBytes = l.smem;
+        cfg.stream = q;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int nclusters = 0;
         NN_CUDA_TRY(cudaOccupancyMaxActiveClusters(&nclusters, (const void *)k, &cfg));
         if (nclusters < 1) {
             set_error("nn_batch_solve: clusters of %d CTAs cannot be scheduled on this device", C);
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
             return NN_ERR_INVALID_ARG;
         }
-        cfg.gridDim = dim3(C * std::min(count, nclusters));
-        cudaEventRecord(e0, st);
-        NN_CUDA_TRY(cudaLaunchKernelEx(&cfg, k, (const BatchInst *)dinst, (const int *)dorder, count, dnext, ctl,
-                                       o->rtol, o->inner_rtol, 200, dcnt, dsc));
+        cfg.gridDim = dim3(C * std::min(l.count, nclusters));
+        NN_CUDA_TRY(cudaLaunchKernelEx(&cfg, k, (const BatchInst *)dinst, (const int *)(dorder + l.first), l.count, next,
+                                       ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc));
         count_launch();
+        return NN_OK;
+    };
+    cudaEventRecord(ev.e0, st);
+    nn_status lr = NN_OK;
+    for (int q = 0; q < nl && lr == NN_OK; ++q) {
+        cudaStream_t on = st;
+        if (q > 0) {
+            on = sides[q - 1].st;
+            NN_CUDA_TRY(cudaStreamWaitEvent(on, ev.e0, 0));
+        }
+        lr = launch(launches[q], dnext + q, on);
     }
-    cudaEventRecord(e1, st);
+    // joined also after a failed launch: the others use this call's memory
+    for (Side &x : sides) {
+        cudaEventRecord(x.done, x.st);
+        cudaStreamWaitEvent(st, x.done, 0);
+    }
+    cudaEventRecord(ev.e1, st);
+    if (lr != NN_OK) {
+        cudaStreamSynchronize(st);
+        return lr;
+    }
     std::vector<int64_t> hc((size_t)count * kBatchCounters);
     std::vector<double> hs((size_t)2 * count);
     NN_CUDA_TRY(cudaMemcpyAsync(hc.data(), dcnt, sizeof(int64_t) * hc.size(), cudaMemcpyDeviceToHost, st));
@@ -214,9 +334,7 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
     NN_CUDA_TRY(cudaStreamSynchronize(st));
     NN_CUDA_TRY(cudaGetLastError());
     float ms = 0.0f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
+    cudaEventElapsedTime(&ms, ev.e0, ev.e1);
     if (ms_out) *ms_out = ms;
     nn_status worst = NN_OK;
     for (int i = 0; i < count; ++i) {
@@ -272,7 +390,7 @@ nn_status nn_batch_solve(int count, nn_system *const *systems, double *const *c,
         int t = 0, c = 0;
         if (sscanf(e, "%dx%d", &t, &c) == 2 && (t == 128 || t == 256 || t == 512) && c >= 1 && c <= kMaxCluster &&
             (c & (c - 1)) == 0) {
-            shape.tpb = c > 1 ? 256 : t;
+            shape.tpb = c > 1 && t != 512 ? 256 : t;
             shape.cluster = c;
         }
     }
@@ -313,9 +431,9 @@ nn_status nn_batch_autotune(int count, nn_system *const *systems, const nn_solve
     nn_solve_opts t = *o;
     std::vector<BatchShape> cands;
     if (largest <= 8192) {
-        cands = {{256, 1}, {512, 1}, {256, 4}, {256, 8}};
+        cands = {{512, 16}, {256, 1}, {512, 1}, {256, 4}, {256, 8}};
     } else {
-        cands = {{256, 4}, {256, 8}, {256, 16}};
+        cands = {{512, 16}, {512, 8}, {256, 8}, {256, 16}};
     }
     float best = 1e30f;
     BatchShape pick_shape;

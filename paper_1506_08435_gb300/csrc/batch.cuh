@@ -36,13 +36,25 @@ struct BatchInst {
     uint8_t *fm;        // n bytes: face mask of the CG phases
 };
 
+constexpr int kBatchResThreads = 512;
+
+// Shared memory of a CTA with `per` slices at most, of at most `slots` entries
+// each, `vbytes` bytes a value (0 slots: the operator stays in global memory).
+__host__ __device__ __forceinline__ size_t batch_res_table(int64_t per) { return ((size_t)(per + 1) * 4 + 15) / 16 * 16; }
+__host__ __device__ __forceinline__ size_t batch_res_bytes(int64_t per, int64_t slots, int vbytes) {
+    return (size_t)per * slots * (4 + vbytes) + batch_res_table(per) + (size_t)kResVectors * per * 32 * vbytes;
+}
+
 constexpr int kBatchCounters = 9;
 
 // Solves instance `id` with team T; this CTA owns the rows R of it.
-template <int MIXED, int CGV, class Team>
+// RES: with the resident CG phase; its operator (LOCAL: in shared memory at op,
+// entries from e0 on) and its shared memory at res.
+template <int MIXED, int CGV, bool RES = false, bool LOCAL = false, class Team>
 __device__ void solve_instance(Team &T, const Rows &R, const BatchInst &I, int id, unsigned rank, unsigned size,
                                const GpcgCtl &ctl, double rtol, double inner_rtol, int max_ref, int64_t *counters,
-                               double *scalars) {
+                               double *scalars, unsigned char *op = nullptr, unsigned char *res = nullptr,
+                               int64_t e0 = 0) {
     const int64_t n = I.n;
     double *x = I.w64;
     R.each([&](int64_t i) { x[i] = I.c[I.free_node[i]]; });
@@ -60,8 +72,24 @@ __device__ void solve_instance(Team &T, const Rows &R, const BatchInst &I, int i
         GpcgVecs<double> v64{x, w6 + n, w6 + 2 * n, w6 + 3 * n, w6 + 4 * n, w6 + 5 * n, w6 + 6 * n,
                              w6 + 7 * n, w6 + 8 * n, I.b0, I.dinv64, I.fm, w6 + 10 * n};
         MixedStats ms;
-        status = mixed_solve<CGV, CGV, true>(T, R, A, A32, I.lo, I.hi, I.b0, x, v, w + 9 * n, w + 10 * n, w + 11 * n, v64,
+        if constexpr (RES) {
+            const int64_t per = (I.nslices + size - 1) / size, ne = I.sptr[R.s1] - I.sptr[R.s0];
+            v.res_sl = reinterpret_cast<int *>(res);
+            v.res = reinterpret_cast<float *>(res + batch_res_table(per));
+            SellF32DiffResX<LOCAL> Ar;
+            if constexpr (LOCAL)
+                static_cast<SellF32DiffLocal &>(Ar) =
+                    SellF32DiffLocal{n, I.nslices, I.sptr, reinterpret_cast<const int32_t *>(op),
+                                     reinterpret_cast<const float *>(op + ne * 4), I.rsum32, false, e0};
+            else
+                static_cast<SellF32Diff &>(Ar) = A32;
+            status = mixed_solve<CGV, CGV, true>(T, R, A, Ar, I.lo, I.hi, I.b0, x, v, w + 9 * n, w + 10 * n, w + 11 * n,
+                                                 v64, rtol * I.den, inner_rtol, max_ref, ctl.max_spmv,
+                                                 batch_inner_product_cap(n), ctl, ctl, ms);
+        } else {
+            status = mixed_solve<CGV, CGV, true>(T, R, A, A32, I.lo, I.hi, I.b0, x, v, w + 9 * n, w + 10 * n, w + 11 * n, v64,
                                 rtol * I.den, inner_rtol, max_ref, ctl.max_spmv, batch_inner_product_cap(n), ctl, ctl, ms);
+        }
         cnt[1] = ms.spmv64;
         cnt[2] = ms.spmv32;
         cnt[3] = ms.cg;
@@ -79,7 +107,22 @@ __device__ void solve_instance(Team &T, const Rows &R, const BatchInst &I, int i
         c.tol = rtol * I.den;
         c.face_tol = 0.5 * c.tol;
         GpcgStats gs;
-        status = gpcg_solve<Team, SellF64, double, CGV>(T, R, A, Bounds<double>{I.lo, I.hi, nullptr, nullptr}, v, c, gs);
+        const Bounds<double> B{I.lo, I.hi, nullptr, nullptr};
+        if constexpr (RES) {
+            const int64_t per = (I.nslices + size - 1) / size, ne = I.sptr[R.s1] - I.sptr[R.s0];
+            v.res_sl = reinterpret_cast<int *>(res);
+            v.res = reinterpret_cast<double *>(res + batch_res_table(per));
+            SellF64ResX<LOCAL> Ar;
+            if constexpr (LOCAL)
+                static_cast<SellF64Local &>(Ar) =
+                    SellF64Local{n, I.nslices, I.sptr, reinterpret_cast<const int32_t *>(op),
+                                 reinterpret_cast<const double *>(op + ne * 4), I.diag, false, e0};
+            else
+                static_cast<SellF64 &>(Ar) = A;
+            status = gpcg_solve<Team, SellF64ResX<LOCAL>, double, CGV>(T, R, Ar, B, v, c, gs);
+        } else {
+            status = gpcg_solve<Team, SellF64, double, CGV>(T, R, A, B, v, c, gs);
+        }
         x = v.x;
         cnt[1] = gs.spmv;
         cnt[3] = gs.cg;
@@ -146,7 +189,7 @@ __global__ void __launch_bounds__(TPB, MIXED ? 2 : 3) k_batch_cluster(const Batc
     __shared__ double xch[2 * kMaxCluster * kMaxRed];
     __shared__ int s_q;
     const unsigned rank = cluster_rank(), size = cluster_size();
-    ClusterTeam T{&sm, xch, rank, size, 0};
+    ClusterTeam T{&sm, xch, rank, size, 0, TPB / 32, nullptr, nullptr, 0};
     for (;;) {
         if (rank == 0 && threadIdx.x == 0) s_q = (int)atomicAdd(next, 1u);
         T.sync();
@@ -172,6 +215,62 @@ __global__ void __launch_bounds__(TPB, MIXED ? 2 : 3) k_batch_cluster(const Batc
     T.sync();   // no CTA leaves while another may still read its shared memory
 }
 
+// The same with the CG phase's vectors in shared memory (cg_resident.cuh), and
+// with LOCAL the CTA's slices of the operator too: 512 threads, one CTA per SM,
+// clusters of 1 to 16 CTAs (an instance of 20 x 20 on one, of 120 x 120 on 16).
+// Bound like the grid's mid-size solves (cg_resident.cuh), with a cluster's
+// mbarriers and pushed sums (about 600 cycles) in place of the grid barrier
+// (2,500).  Measured: see the rule of the launch shapes in batch.cu.
+template <int MIXED, bool LOCAL>
+__global__ void __launch_bounds__(kBatchResThreads, 1) k_batch_res(const BatchInst *__restrict__ insts,
+                                                                  const int *__restrict__ order, int count,
+                                                                  unsigned *next, GpcgCtl ctl, double rtol,
+                                                                  double inner_rtol, int max_ref, int64_t *counters,
+                                                                  double *scalars) {
+    __shared__ RedSmem sm;
+    __shared__ double xch[2 * kMaxCluster * kMaxRed];
+    __shared__ double rx[2 * 3 * kMaxCluster];
+    __shared__ uint64_t mb[4];
+    __shared__ int s_q, s_q0;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    const unsigned rank = cluster_rank(), size = cluster_size();
+    ClusterTeam T{&sm, xch, rank, size, 0, 1, mb, rx, 0};
+    if (threadIdx.x == 0) T.res_init();
+    for (;;) {
+        if (rank == 0 && threadIdx.x == 0) s_q = (int)atomicAdd(next, 1u);
+        T.sync();
+        // every CTA reads the instance index taken by CTA 0
+        if (threadIdx.x == 0) {
+            int q;
+            asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(q) : "r"(ClusterTeam::remote(&s_q, 0)) : "memory");
+            s_q0 = q;
+        }
+        T.sync();
+        if (s_q0 >= count) break;
+        const int id = order[s_q0];
+        const BatchInst I = insts[id];
+        const Rows R = rows_of_block(I.n, I.nslices, (int)rank, (int)size);
+        T.active = R.active_warps(kBatchResThreads / 32);
+        const int64_t per = (I.nslices + size - 1) / size, e0 = I.sptr[R.s0], ne = I.sptr[R.s1] - e0;
+        const int vbytes = MIXED ? 4 : 8;
+        unsigned char *at = dyn;
+        if constexpr (LOCAL) {
+            const int4 *gc = reinterpret_cast<const int4 *>(I.col + e0);
+            const int4 *gv = MIXED ? reinterpret_cast<const int4 *>(I.val32 + e0) : reinterpret_cast<const int4 *>(I.val + e0);
+            for (int64_t q = threadIdx.x; q < ne / 4; q += blockDim.x) reinterpret_cast<int4 *>(dyn)[q] = __ldg(gc + q);
+            for (int64_t q = threadIdx.x; q < ne * vbytes / 16; q += blockDim.x)
+                reinterpret_cast<int4 *>(dyn + ne * 4)[q] = __ldg(gv + q);
+            at += ne * (4 + vbytes);
+        }
+        GpcgCtl c = ctl;
+        c.res_warps = resident_warps(per);
+        solve_instance<MIXED, 2, true, LOCAL>(T, R, I, id, rank, size, c, rtol, inner_rtol, max_ref, counters, scalars,
+                                              dyn, at, e0);
+        T.sync();
+    }
+    T.sync();   // no CTA leaves while another may still read its shared memory
+}
+
 using BatchKernel = void (*)(const BatchInst *, const int *, int, unsigned *, GpcgCtl, double, double, int,
                              int64_t *, double *);
 
@@ -180,5 +279,8 @@ using BatchKernel = void (*)(const BatchInst *, const int *, int, unsigned *, Gp
 // that combination is not built.
 BatchKernel batch_kernel_fp64(int tpb, int cluster, int cgv);
 BatchKernel batch_kernel_mixed(int tpb, int cluster, int cgv);
+// k_batch_res, any cluster size.
+BatchKernel batch_res_kernel_fp64(bool local);
+BatchKernel batch_res_kernel_mixed(bool local);
 
 }  // namespace nnqp

@@ -16,9 +16,10 @@
 //   * few compute warps with several slices each: a thread's rows are added by
 //     the dot products' own FMAs, and the tree over the block has 4-12 warps;
 //   * the two things that every block waits for are apart and hidden.  m goes
-//     out first and its barrier (counter count2, warp 12) runs while the other
+//     out first and its barrier (warp 12; the grid's counter count2, or a
+//     cluster's mbarriers) runs while the other
 //     five recurrences and the dot products are computed; the sums and the
-//     scalar step (warps 13-15, counter count) run while the next product is
+//     scalar step (warps 13-15) run while the next product is
 //     computed, which needs m only.
 // The product of the iteration after the last one is thus computed and not
 // used (one per phase; it is counted).
@@ -136,11 +137,11 @@ __device__ __forceinline__ void resident_product(const Op &A, const int *sl, boo
 // block calls it; na compute warps.  Returns 0, ST_TIMEOUT when a wait gave
 // up, or 1 when the face has nothing to reduce.  A call of its own: the
 // registers the caller keeps live are saved once per phase.
-template <class Op, typename V>
-__device__ __noinline__ int cg_resident(GridTeam &T_, const Rows &R_, const Op &A_, const Bounds<V> &B,
+template <class Team, class Op, typename V>
+__device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, const Bounds<V> &B,
                                         const GpcgVecs<V> &v_, const GpcgCtl &C_, GpcgStats &st, double ftol2,
                                         int na) {
-    GridTeam T = T_;
+    Team T = T_;
     const Rows R = R_;
     Op A = A_;
     if constexpr (IsResidentOp<Op>::local) {
@@ -279,7 +280,8 @@ __device__ __noinline__ int cg_resident(GridTeam &T_, const Rows &R_, const Op &
         for (;;) {
             named_sync(1, n1);
             ++it;
-            if (lane == 0) sm.flag2[it & 1] = T.arrive_and_wait_on(&T.bar->count2, T.wait2 + it);
+            const int ok = T.res_vector_barrier(it);
+            if (lane == 0) sm.flag2[it & 1] = ok;
             __syncwarp();
             named_arrive(2, n1);
             named_sync(4, n4);
@@ -291,26 +293,22 @@ __device__ __noinline__ int cg_resident(GridTeam &T_, const Rows &R_, const Op &
         // on a warp (and sub-core) each: warp 13 alpha, 14 beta and 1 / gamma,
         // 15 the test.  (One warp after the other it took 1,850 cycles.)
         const int k = warp - (kResWarps + 1);
-        int slot = T.slot;
         double t = cs.igamma * cs.ialpha;                          // warp 13
         double ig = cs.igamma;                                     // warp 14
         double dec = 0.5 * cs.alpha * cs.gamma, maxdec = dec;      // warp 15
         for (;;) {
-            slot ^= 1;
             ++it;
-            double *P = T.partials + (size_t)slot * kMaxRed * T.nblocks;
             double *sc = sm.sc + 8 * (it & 1);
             if (k == 0) {
                 named_sync(3, n1);
                 warp0_sum_warps<3>(sm, na);
                 __syncwarp();
-                if (lane < 3) P[(size_t)lane * T.nblocks + blockIdx.x] = sm.bcast[lane];
-                __syncwarp();
-                if (lane == 0) sm.flag = T.arrive_and_wait_on(&T.bar->count, T.wait_id + it);
+                const int ok = T.res_publish(it);
+                if (lane == 0) sm.flag = ok;
                 __syncwarp();
             }
             named_sync(5, 96);
-            const double sum = sm.flag ? sum_partials(P + (size_t)k * T.nblocks, T.nblocks) : 0.0;
+            const double sum = sm.flag ? T.res_sum(k, it) : 0.0;
             if (lane == 0) sm.bcast[8 + k] = sum;
             named_sync(5, 96);
             const double gamma = sm.bcast[8];
@@ -352,9 +350,7 @@ __device__ __noinline__ int cg_resident(GridTeam &T_, const Rows &R_, const Op &
     it = sm.its;
     if (it < 0) return ST_TIMEOUT;
     T_ = T;
-    T_.slot ^= it & 1;
-    T_.wait_id += it;
-    T_.wait2 += it;
+    T_.res_end(it);
     st.spmv += it + 1;
     st.cg += it;
     st.fl += 20 * (int64_t)it;

@@ -242,8 +242,8 @@ struct GpcgStats {
     double gp2 = 0.0;
 };
 
-template <class Op, typename V>
-__device__ __noinline__ int cg_resident(GridTeam &T, const Rows &R, const Op &A, const Bounds<V> &B,
+template <class Team, class Op, typename V>
+__device__ __noinline__ int cg_resident(Team &T, const Rows &R, const Op &A, const Bounds<V> &B,
                                         const GpcgVecs<V> &v, const GpcgCtl &C, GpcgStats &st, double ftol2, int na);
 
 // Runs GPCG from the iterate in v.x (projected first).  On exit v.x holds
@@ -368,13 +368,13 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
         if (st.gp2 <= tol2 || st.spmv >= C.max_spmv || !isfinite(st.gp2)) continue;
         // ------------------------------------------------ CG on faces
         const bool count_cross = C.cg_bound_stop != 0;
-        constexpr bool can_reside = CGV == 2 && IsResidentOp<Op>::value && IsGridTeam<Team>::value;
+        constexpr bool can_reside = CGV == 2 && IsResidentOp<Op>::value;
         for (;;) {
             if (can_reside && C.res_warps > 0) {
                 if constexpr (can_reside) {
                     // (copies for the call: what is passed by reference lives in the
                     // stack frame, and the passes here would reload it at every use)
-                    GridTeam t = T;
+                    Team t = T;
                     GpcgStats s = st;
                     const Rows r = R;
                     const Op a = A;

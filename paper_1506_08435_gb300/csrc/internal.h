@@ -137,6 +137,7 @@ struct nn_system {
     nnqp::SsorF64 ssor{};           // SSOR ordering (ncolors = 0 until nn_precond_setup)
     int64_t ssor_slices = 0;
     std::vector<int32_t> ssor_color; // colour of each free unknown (host)
+    int64_t max_slice_slots = 0;    // entries of the widest SELL slice
     double anorm_inf = 0;           // ||A||_inf
     double b0norm = 0;              // ||b0||_2
     bool has_csr = false, has_mixed = false, has_full = false;

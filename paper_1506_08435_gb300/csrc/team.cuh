@@ -289,6 +289,34 @@ struct GridTeam {
         return ok;
     }
 
+    // What the resident CG phase (cg_resident.cuh) waits for, by event number
+    // it = 1, 2, ... of the phase; each is called by all lanes of one warp and
+    // returns 1, or 0 when the wait gave up.
+    // m of every block visible:
+    __device__ int res_vector_barrier(int it) {
+        int ok = 1;
+        if ((threadIdx.x & 31) == 0) ok = arrive_and_wait_on(&bar->count2, wait2 + it);
+        return __shfl_sync(0xffffffffu, ok, 0);
+    }
+    // the block's three sums (sm->bcast) published, everybody's there:
+    __device__ int res_publish(int it) {
+        const int lane = threadIdx.x & 31;
+        if (lane < 3) res_partials(it)[(size_t)lane * nblocks + blockIdx.x] = sm->bcast[lane];
+        __syncwarp();
+        int ok = 1;
+        if (lane == 0) ok = arrive_and_wait_on(&bar->count, wait_id + it);
+        return __shfl_sync(0xffffffffu, ok, 0);
+    }
+    // sum k over the blocks:
+    __device__ double res_sum(int k, int it) { return sum_partials(res_partials(it) + (size_t)k * nblocks, nblocks); }
+    __device__ double *res_partials(int it) { return partials + (size_t)(slot ^ (it & 1)) * kMaxRed * nblocks; }
+    // after a phase of `it` events
+    __device__ void res_end(int it) {
+        slot ^= it & 1;
+        wait_id += it;
+        wait2 += it;
+    }
+
     __device__ bool sync() {
         __syncthreads();
         ++wait_id;
@@ -364,15 +392,6 @@ struct GridTeam {
     }
 };
 
-template <class Team>
-struct IsGridTeam {
-    static constexpr bool value = false;
-};
-template <>
-struct IsGridTeam<GridTeam> {
-    static constexpr bool value = true;
-};
-
 constexpr int kMaxCluster = 16;
 
 // The CTAs of one thread-block cluster (all co-scheduled by the hardware).
@@ -387,6 +406,72 @@ struct ClusterTeam {
     double *xch;                  // this CTA's [2][kMaxCluster][kMaxRed] exchange buffer (shared memory)
     unsigned rank, size;
     int slot;
+    int active;                   // warps of this CTA that own rows
+    uint64_t *mb;                 // resident CG phase: mbarriers, [0..1] m written, [2..3] sums (shared memory)
+    double *rx;                   //   sums received, [2][3][kMaxCluster]
+    int events;                   //   events passed (each uses the mbarriers of its parity)
+
+    // The resident CG phase's waits (see GridTeam).  Each event uses one of two
+    // mbarriers in turn: a CTA can be one event ahead of another, never two.
+    __device__ static uint32_t remote(const void *p, unsigned r) {
+        uint32_t a;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(r));
+        return a;
+    }
+    __device__ static int wait_cluster(uint64_t *b, unsigned parity) {
+        for (int it = 0; it < (1 << 22); ++it) {
+            unsigned done;
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], "
+                "%2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done)
+                : "r"((uint32_t)__cvta_generic_to_shared(b)), "r"(parity)
+                : "memory");
+            if (done) return 1;
+        }
+        return 0;
+    }
+    __device__ void res_init() {   // by one thread, before a cluster barrier
+        for (int k = 0; k < 4; ++k)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(mb + k)),
+                         "r"(k < 2 ? size : 1u)
+                         : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __device__ int res_vector_barrier(int it) {
+        const unsigned e = (unsigned)(events + it), lane = threadIdx.x & 31;
+        uint64_t *b = mb + (e & 1);
+        if (lane < size)
+            asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote(b, lane))
+                         : "memory");
+        __syncwarp();
+        return __all_sync(0xffffffffu, wait_cluster(b, ((e - 1) >> 1) & 1));
+    }
+    __device__ int res_publish(int it) {
+        const unsigned e = (unsigned)(events + it), lane = threadIdx.x & 31;
+        uint64_t *b = mb + 2 + (e & 1);
+        if (lane == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(b)),
+                         "r"(size * 24u)
+                         : "memory");
+        for (unsigned q = lane; q < size * 3; q += 32) {
+            const unsigned r = q / 3, k = q - 3 * r;
+            asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u64 [%0], %1, [%2];" ::"r"(
+                             remote(rx + ((e & 1) * 3 + k) * kMaxCluster + rank, r)),
+                         "l"(__double_as_longlong(sm->bcast[k])), "r"(remote(b, r))
+                         : "memory");
+        }
+        __syncwarp();
+        return __all_sync(0xffffffffu, wait_cluster(b, ((e - 1) >> 1) & 1));
+    }
+    __device__ double res_sum(int k, int it) {
+        const unsigned e = (unsigned)(events + it), lane = threadIdx.x & 31;
+        double u = lane < size ? rx[((e & 1) * 3 + k) * kMaxCluster + lane] : 0.0;
+        for (int o = (int)size >> 1; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+        return u;
+    }
+    __device__ void res_end(int it) { events += it; }
 
     __device__ __forceinline__ static void cluster_barrier() {
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
@@ -399,12 +484,12 @@ struct ClusterTeam {
     template <int K>
     __device__ bool reduce(double (&v)[K]) {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        warp_stage<K>(v, *sm);
+        if (warp < active) warp_stage<K>(v, *sm);
         __syncthreads();
         slot ^= 1;
         double *buf = xch + (size_t)slot * kMaxCluster * kMaxRed;
         if (warp == 0) {
-            warp0_sum_warps<K>(*sm, nw);
+            warp0_sum_warps<K>(*sm, active);
             __syncwarp();
             for (int q = lane; q < (int)size * K; q += 32) {
                 const unsigned r = (unsigned)(q / K);
