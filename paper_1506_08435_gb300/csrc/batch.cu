@@ -225,8 +225,8 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
     ctl.max_spmv = o->max_iter;
     ctl.gp_max = 50;
     ctl.cg_max = 1 << 30;
-    ctl.eta1 = 0.1;
-    ctl.eta2 = 1e-3;
+    ctl.eta1 = kEta1;
+    ctl.eta2 = kEta2;
     ctl.mu = 1e-4;
     ctl.cg_variant = 0;
     ctl.cg_bound_stop = 0;

@@ -48,10 +48,6 @@ constexpr int kResVectors = 9;        // vectors of the block's rows in shared m
 // three slices a warp, then 12; 4 where a warp has one slice at most.
 __host__ __device__ __forceinline__ int resident_warps(int64_t per) { return per <= 4 ? 4 : per <= 24 ? 8 : 12; }
 
-// x != 0 without a floating-point comparison (FP64 ones hold the FP64 unit).
-__device__ __forceinline__ bool is_set(double x) { return __double_as_longlong(x) != 0; }
-__device__ __forceinline__ bool is_set(float x) { return __float_as_int(x) != 0; }
-
 __device__ __forceinline__ void named_sync(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
@@ -175,7 +171,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
             if (l < n) {
                 const int64_t i = base + l;
                 const V xi = v.x[i];
-                if (xi > B.l(i) && xi < B.h(i)) {
+                if (num_lt(B.l(i), xi) && num_lt(xi, B.h(i))) {
                     dl = v.dinv[i];
                     ri = -v.g[i];
                     ui = dl * ri;

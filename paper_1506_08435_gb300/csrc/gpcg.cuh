@@ -41,6 +41,29 @@ enum : int {
     ST_TIMEOUT = 7,
 };
 
+// FP64 comparisons hold the FP64 unit as long as a multiply-add (64 cycles of a
+// sub-core per warp instruction), and the projections make ten of them per row.
+// These give the same answers, NaN included, on the integer units.
+__device__ __forceinline__ long long order_key(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);   // ascending with x (-0 just below +0)
+}
+__device__ __forceinline__ bool not_nan(double x) {
+    return (unsigned long long)(__double_as_longlong(x) << 1) <= 0xffe0000000000000ULL;
+}
+__device__ __forceinline__ bool num_lt(double x, double y) {
+    const long long a = order_key(x), b = order_key(y);
+    // (a zero of either sign is not below the other)
+    return a < b && not_nan(x) && not_nan(y) && ((__double_as_longlong(x) | __double_as_longlong(y)) << 1) != 0;
+}
+__device__ __forceinline__ bool num_le(double x, double y) {
+    const long long a = order_key(x), b = order_key(y);
+    return not_nan(x) && not_nan(y) &&
+           (a <= b || ((__double_as_longlong(x) | __double_as_longlong(y)) << 1) == 0);
+}
+__device__ __forceinline__ bool num_lt(float x, float y) { return x < y; }
+__device__ __forceinline__ bool num_le(float x, float y) { return x <= y; }
+
 template <typename V>
 struct Bounds {
     double lo, hi;
@@ -52,17 +75,26 @@ struct Bounds {
 
 template <typename V>
 __device__ __forceinline__ V clampv(V x, V l, V h) {
-    return x < l ? l : (x > h ? h : x);
+    return num_lt(x, l) ? l : (num_lt(h, x) ? h : x);
 }
+
+template <typename V>
+__device__ __forceinline__ bool at_bound(V x, V l, V h) {
+    return num_le(x, l) || num_le(h, x);
+}
+
+// x != 0 (a NaN is)
+__device__ __forceinline__ bool is_set(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ bool is_set(float x) { return x != 0.0f; }
 
 // Projected gradient of the box QP at x.
 template <typename V>
 __device__ __forceinline__ V proj_grad(V x, V g, V l, V h) {
-    if (x <= l) {
-        if (x >= h) return (V)0;
-        return g < (V)0 ? g : (V)0;
+    if (num_le(x, l)) {
+        if (num_le(h, x)) return (V)0;
+        return num_lt(g, (V)0) ? g : (V)0;
     }
-    if (x >= h) return g > (V)0 ? g : (V)0;
+    if (num_le(h, x)) return num_lt((V)0, g) ? g : (V)0;
     return g;
 }
 
@@ -212,13 +244,27 @@ struct GpcgVecs {
     int *res_sl;          //    and the first entries of its slices
 };
 
+constexpr double kEta1 = 0.3, kEta2 = 0.06;           // steady solves
+constexpr double kEta1Warm = 0.1, kEta2Warm = 1e-3;   // time steps
+
 struct GpcgCtl {
     double tol;          // stop when ||gP||_2 <= tol
     double face_tol;     // CG stops when the face residual norm <= face_tol
     int64_t max_spmv;    // cap on products for this call
     int gp_max;          // gradient-projection steps per phase
     int cg_max;          // CG iterations per face
-    double eta1, eta2;   // stall ratios of the GP and CG phases
+    // Stall ratios of the GP and CG phases: a phase ends when a step decreases
+    // the objective by less than that share of the phase's best step.  On a face
+    // that is not yet the solution's, what CG gains late in a phase is clipped
+    // away by the projected search, so steady solves from afar leave it early
+    // (kEta1, kEta2); a warm-started time step starts near its face and leaves it
+    // late.  Products with (0.1, 1e-3) / (0.3, 0.06): 397 x 283 78,140 / 47,756,
+    // 173 x 173 29,487 / 21,830, 120 x 120 11,456 / 7,502 (three problems each);
+    // 44^3 15,146 / 10,679, 70^3 15,695 / 11,007, 90^3 mixed 20,360 / 14,705; 16
+    // batch instances 52,410 / 43,279; cube with a hole, m = 4 2,030 / 1,837 (m =
+    // 2 889 / 891, its 6% longer); 40^3 transient in time 19.7 / 20.3 ms.  With
+    // 0.1 for the second the cubes with a hole lose 5 to 18%, the others gain 3%.
+    double eta1, eta2;
     double mu;           // Armijo constant
     int cg_variant;      // 0: textbook PCG (3 team barriers per iteration);
                          // 1: Chronopoulos-Gear PCG (2 barriers, one fused reduction);
@@ -316,7 +362,7 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
                     V wi = clampv(xi - va * proj_grad(xi, v.g[i], l, h), l, h);
                     v.w[i] = wi;
                     a2[0] += v.g[i] * (wi - xi);
-                    a2[1] += ((xi <= l || xi >= h) != (wi <= l || wi >= h)) ? one : zero;
+                    a2[1] += (at_bound(xi, l, h) != at_bound(wi, l, h)) ? one : zero;
                 });
                 if (!T.sync()) return ST_TIMEOUT;
                 A.apply(R, v.w, [&](int64_t i, V aw) {
@@ -393,7 +439,7 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
                 // product A p carried by the recurrence q = w + beta q.
                 R.each([&](int64_t i) {
                     V xi = v.x[i];
-                    const bool fr = xi > B.l(i) && xi < B.h(i);
+                    const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
                     v.fm[i] = fr ? 1 : 0;
                     V ri = fr ? -v.g[i] : zero;
                     v.r[i] = ri;
@@ -480,7 +526,7 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
                 V *mc = v.gw, *mn = v.m2;
                 R.each([&](int64_t i) {
                     V xi = v.x[i];
-                    const bool fr = xi > B.l(i) && xi < B.h(i);
+                    const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
                     v.fm[i] = fr ? 1 : 0;
                     V ri = fr ? -v.g[i] : zero;
                     v.r[i] = ri;
@@ -565,7 +611,7 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
                 if constexpr (PC) {
                     R.each([&](int64_t i) {
                         V xi = v.x[i];
-                        const bool fr = xi > B.l(i) && xi < B.h(i);
+                        const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
                         v.fm[i] = fr ? 1 : 0;
                         v.r[i] = fr ? -v.g[i] : zero;
                         v.s[i] = zero;
@@ -583,7 +629,7 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
                 } else {
                     R.each([&](int64_t i) {
                         V xi = v.x[i];
-                        const bool fr = xi > B.l(i) && xi < B.h(i);
+                        const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
                         v.fm[i] = fr ? 1 : 0;
                         V ri = fr ? -v.g[i] : zero;
                         V zi = v.dinv[i] * ri;
@@ -757,7 +803,7 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
                     a6[2] += (v.g[i] + gwi) * (wi - v.x[i]);
                     V gp = proj_grad(wi, gwi, l, h);
                     a6[3] += gp * gp;
-                    a6[4] += ((wi <= l || wi >= h) && gp != zero) ? one : zero;
+                    a6[4] += (at_bound(wi, l, h) && is_set(gp)) ? one : zero;
                 });
                 // Armijo test; after acceptance the face loop ends on convergence
                 // or on a non-binding active entry (back to gradient projection)

@@ -195,6 +195,9 @@ constexpr size_t kTmaSmemBytes = 196 * 1024;
 // the large mixed grid where the streamed operator does not apply.
 constexpr int kLargeThreads = 768;
 constexpr int kLargeThreadsLoads = 512;
+// Unknowns of an FP64 system from which that grid beats one 512-thread block
+// per SM with CG form 1 (between 80^3 and 96^3).
+constexpr int64_t kWideRows = 640000;
 // Threads per block of the projected L-BFGS kernel (128 was measured too:
 // faster on the 50^2 problem, slower on the 40^3 transient run).
 constexpr int kLbfgsThreads = 256;
@@ -373,8 +376,11 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     // need the long phases
     a.ctl.gp_max = mode_transient(mode) ? 3 : 50;
     a.ctl.cg_max = 1 << 30;
-    a.ctl.eta1 = 0.1;
-    a.ctl.eta2 = 1e-3;
+    // (a served 3D solution, which the default tolerance leaves open by 1e-9, has
+    // to be the same bits from release to release: it keeps the late ratios)
+    const bool late = mode_transient(mode) || (force_tpb != 0 && s->dim == 3);
+    a.ctl.eta1 = late ? kEta1Warm : kEta1;
+    a.ctl.eta2 = late ? kEta2Warm : kEta2;
     a.ctl.mu = 1e-4;
     // CG form: the pipelined one (one barrier per iteration) where barrier
     // latency bounds the solve; the textbook one on large systems, where the
@@ -455,9 +461,26 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     // blocks measure alike there).  Served solves (force_tpb) do without: blocks
     // of several requests share an SM, which its shared memory would not allow,
     // and what a request returns stays the same bits.
+    // Between those and 2^20 unknowns the best form and block depend on how
+    // much of an SM's time is FP64 and how much barrier (us per product, form 2
+    // x 3 blocks of 256 / form 1 x 512 / form 0 x 768 threads, steady FP64): 56^3
+    // 18.6 / 17.0 / 20.9, 72^3 32.4 / 27.5 / 32.1, 80^3 41.0 / 35.5 / 38.9, 96^3
+    // 65.6 / 68.2 / 58.7; mixed, 768 threads with the streamed FP32 operator
+    // where it exceeds 48 MB: 56^3 18.7 / 12.7 / 17.8, 72^3 31.8 / 27.5 / 28.5,
+    // 80^3 32.0 / 29.6 / 28.1, 96^3 49.7 / 46.1 / 36.1.
+    bool wide = false;   // one 512-thread block per SM
+    if (large && !force_large && force_tpb == 0 && fmt == NN_FMT_SELL && a.ctl.cg_variant == 2 &&
+        !getenv("NNQP_CG_VARIANT")) {
+        if (mixed ? !a.A32.stream : n < kWideRows) {
+            a.ctl.cg_variant = 1;
+            wide = true;
+        } else if (mixed || mode == MODE_STEADY) {
+            a.ctl.cg_variant = 0;
+        }
+    }
     const bool mid = !driver && !large && slices <= (int64_t)4 * 8 * sms;
     const bool on_chip = mid && force_tpb == 0 && fmt == NN_FMT_SELL && a.ctl.cg_variant == 2 && mode != MODE_MIXED;
-    if (mid && (on_chip || slices > (int64_t)8 * sms / 2)) tpb = 512;
+    if (wide || (mid && (on_chip || slices > (int64_t)8 * sms / 2))) tpb = 512;
     if (!driver && (force_tpb == 256 || force_tpb == 512)) tpb = force_tpb;
     if (large && (a.ctl.cg_variant == 0 || a.ctl.cg_variant == 3) && fmt == NN_FMT_SELL && force_tpb != 512)
         tpb = kLargeThreads;

@@ -179,7 +179,7 @@ __device__ int tron_solve(Team &T, const Rows &R, const Op &A, const Bounds<doub
             if (v.pc) {
                 R.each([&](int64_t i) {
                     const double xi = v.x[i];
-                    const bool fr = xi > B.l(i) && xi < B.h(i);
+                    const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
                     v.fm[i] = fr ? 1 : 0;
                     const double ri = fr ? -v.g[i] : 0.0;
                     v.r[i] = ri;
@@ -198,7 +198,7 @@ __device__ int tron_solve(Team &T, const Rows &R, const Op &A, const Bounds<doub
             } else {
                 R.each([&](int64_t i) {
                     const double xi = v.x[i];
-                    const bool fr = xi > B.l(i) && xi < B.h(i);
+                    const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
                     v.fm[i] = fr ? 1 : 0;
                     const double ri = fr ? -v.g[i] : 0.0;
                     const double zi = v.dinv[i] * ri;
@@ -320,7 +320,7 @@ __device__ int tron_solve(Team &T, const Rows &R, const Op &A, const Bounds<doub
                     a3[1] += (v.g[i] + gwi) * (wi - xi);
                     const double gp = proj_grad(wi, gwi, l, h);
                     a3[2] += gp * gp;
-                    a3[3] += ((wi <= l || wi >= h) && xi > l && xi < h) ? 1.0 : 0.0;   // newly active
+                    a3[3] += (at_bound(wi, l, h) && num_lt(l, xi) && num_lt(xi, h)) ? 1.0 : 0.0;   // newly active
                 });
                 double o3[1];
                 if (!team_sum_scalar(T, a3, d3, o3, [&](const double (&s)[4], double (&r)[1]) {
