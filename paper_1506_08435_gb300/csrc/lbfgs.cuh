@@ -93,10 +93,21 @@ __device__ int lbfgs_solve(Team &T, const Rows &R, const Op &A, double lo, doubl
         // ---- model coefficients from u = S'gP, v = Y'gP (carried over)
         bool use_model = k > 0;
         if (use_model) {
-            if (threadIdx.x == 0) {
+            if (threadIdx.x < 32) {
                 const double gamma = sm.SY[(k - 1) * kLbfgsMax + (k - 1)] / sm.YY[(k - 1) * kLbfgsMax + (k - 1)];
-                sm.ok = lbfgs_coefficients(k, sm.SY, sm.YY, uv, uv + kLbMaxM, gamma, sm.cs, sm.cy) ? 1 : 0;
-                sm.cs[kLbfgsMax - 1] = gamma;
+                const int l = (int)threadIdx.x < k ? (int)threadIdx.x : 0;
+                double ul = uv[0], vl = uv[kLbMaxM];
+#pragma unroll
+                for (int j = 1; j < kLbMaxM; ++j)
+                    if (j == l) {
+                        ul = uv[j];
+                        vl = uv[kLbMaxM + j];
+                    }
+                const bool ok = lbfgs_coefficients_warp(k, sm.SY, sm.YY, ul, vl, gamma, sm.cs, sm.cy);
+                if (threadIdx.x == 0) {
+                    sm.ok = ok ? 1 : 0;
+                    sm.cs[kLbfgsMax - 1] = gamma;
+                }
             }
             __syncthreads();
             use_model = sm.ok != 0;
@@ -104,7 +115,7 @@ __device__ int lbfgs_solve(Team &T, const Rows &R, const Op &A, double lo, doubl
         // ---- projected backtracking search along d = -H gP (zero on the binding set)
         double alpha = 1.0;
         bool accepted = false, have_d = false;
-        double a[kLbW];
+        double a[kLbW], o[3];   // o: descent direction, decrease enough, pair good
         for (int ls = 0; ls < 60; ++ls) {
 #pragma unroll
             for (int q = 0; q < kLbW; ++q) a[q] = 0.0;
@@ -160,12 +171,18 @@ __device__ int lbfgs_solve(Team &T, const Rows &R, const Op &A, double lo, doubl
                         a[LB_X + 4 * kLbMaxM + j] += yj * gp;
                     }
             });
-            if (!T.reduce(a)) return ST_TIMEOUT;
+            // the tests once per block (a root by every warp holds the FP64 units)
+            if (!team_sum_scalar_d(T, a, o, [&](const double (&s)[kLbW], double (&r)[3]) {
+                    r[0] = s[LB_GD] < 0.0 ? 1.0 : 0.0;
+                    r[1] = 0.5 * s[LB_QD] <= C.mu * s[LB_GDX] ? 1.0 : 0.0;
+                    r[2] = s[LB_SY] > 1e-12 * sqrt(s[LB_SS] * s[LB_YY]) ? 1.0 : 0.0;
+                }))
+                return ST_TIMEOUT;
             ++st.spmv;
             st.vec += 6 + 2 * k + 3;
             if (first) {
                 have_d = true;
-                if (!(a[LB_GD] < 0.0)) {
+                if (!flag_set(o[0])) {
                     if (!use_model) return ST_NUMERIC;
                     use_model = false;   // not a descent direction: drop the memory
                     k = 0;
@@ -174,7 +191,7 @@ __device__ int lbfgs_solve(Team &T, const Rows &R, const Op &A, double lo, doubl
                     continue;
                 }
             }
-            if (0.5 * a[LB_QD] <= C.mu * a[LB_GDX]) {
+            if (flag_set(o[1])) {
                 accepted = true;
                 break;
             }
@@ -186,7 +203,7 @@ __device__ int lbfgs_solve(Team &T, const Rows &R, const Op &A, double lo, doubl
         t = g; g = gw; gw = t;
         st.gp2 = a[LB_GP2];
         // ---- memory update; uv follows the pairs to their new positions
-        if (a[LB_SY] > 1e-12 * sqrt(a[LB_SS] * a[LB_YY])) {
+        if (flag_set(o[2])) {
             const int drop = k == m ? 1 : 0;
             if (threadIdx.x == 0) {
                 // new dots indexed by the old positions j; after a drop old j maps to j - 1

@@ -55,4 +55,38 @@ NN_HD inline bool lbfgs_coefficients(int k, const double *SY, const double *YY, 
     return true;
 }
 
+#if defined(__CUDACC__)
+// The same by one warp, lane i for row i (every lane calls it; u, v: the lane's
+// entries).  One thread took some 9,000 cycles for k = 5, an FP64 operation being
+// 64; here the divisions and the rows of w go side by side and a substitution
+// step is one multiplication, one broadcast and one multiply-add.
+__device__ inline bool lbfgs_coefficients_warp(int k, const double *SY, const double *YY, double u, double v,
+                                               double gamma, double *cs, double *cy) {
+    const unsigned all = 0xffffffffu;
+    const int i = threadIdx.x & 31;
+    const bool in = i < k;
+    const double rii = in ? SY[i * kLbfgsMax + i] : 1.0;
+    if (!__all_sync(all, rii > 0.0)) return false;
+    const double rinv = 1.0 / rii;
+    double s = in ? u : 0.0, t = 0.0;
+    for (int j = k - 1; j >= 0; --j) {       // R t = u
+        const double tj = __shfl_sync(all, s * rinv, j);
+        if (i == j) t = tj;
+        if (i < j) s -= SY[i * kLbfgsMax + j] * tj;
+    }
+    double w = in ? rii * t - gamma * v : 0.0;   // w = (D + gamma Y^T Y) t - gamma v
+    for (int j = 0; j < k; ++j) {
+        const double tj = __shfl_sync(all, t, j);
+        if (in) w += gamma * YY[i * kLbfgsMax + j] * tj;
+    }
+    for (int j = 0; j < k; ++j) {            // R^T p = w
+        const double pj = __shfl_sync(all, w * rinv, j);
+        if (i == j) cs[j] = pj;
+        if (in && i > j) w -= SY[j * kLbfgsMax + i] * pj;
+    }
+    if (in) cy[i] = -gamma * t;
+    return true;
+}
+#endif
+
 }  // namespace nnqp

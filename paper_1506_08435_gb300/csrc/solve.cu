@@ -14,13 +14,30 @@
 
 namespace nnqp {
 
-// The same driver with the projected L-BFGS solver (FP64, SELL).
+// Copies the entries of the block's slices of the FP64 operator to shared
+// memory at dst (columns, then values).
+__device__ __forceinline__ SellF64Local stage_operator(const SellF64 &A, const Rows &R, unsigned char *dst) {
+    const int64_t e0 = A.sptr[R.s0], ne = A.sptr[R.s1] - e0;   // a multiple of 64
+    const int4 *gc = reinterpret_cast<const int4 *>(A.col + e0), *gv = reinterpret_cast<const int4 *>(A.val + e0);
+    for (int64_t q = threadIdx.x; q < ne / 4; q += blockDim.x) reinterpret_cast<int4 *>(dst)[q] = __ldg(gc + q);
+    for (int64_t q = threadIdx.x; q < ne / 2; q += blockDim.x) reinterpret_cast<int4 *>(dst + ne * 4)[q] = __ldg(gv + q);
+    return SellF64Local{A.n, A.nslices, A.sptr, reinterpret_cast<const int32_t *>(dst),
+                        reinterpret_cast<const double *>(dst + ne * 4), A.diag, false, e0};
+}
+
+// The same driver with the projected L-BFGS solver (FP64, SELL).  LOCAL as for
+// TRON below, in 256-thread blocks (its product keeps 39 sums a thread).
+template <bool LOCAL>
 __global__ void __launch_bounds__(kSolveThreads) k_lbfgs_grid(GridArgs a) {
     __shared__ RedSmem sm;
     __shared__ LbSmem lsm;
+    extern __shared__ __align__(16) unsigned char drv_smem[];
     GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm, 0, 0};
     const Rows R = rows_of_block(a.n, a.nslices, blockIdx.x, gridDim.x);
     T.active = R.active_warps(blockDim.x >> 5);
+    SellF64X<LOCAL> A;
+    if constexpr (LOCAL) A = stage_operator(a.A, R, drv_smem);
+    else A = a.A;
     double *x0 = a.v64[0];
     R.each([&](int64_t i) { x0[i] = a.c_in[a.free_node[i]]; });
     if (!T.sync()) return;
@@ -38,7 +55,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_lbfgs_grid(GridArgs a) {
         double *x = x0, *g = a.v64[1], *w = a.v64[7], *gw = a.v64[8];
         LbCtl c{a.rtol * den, a.ctl.max_spmv, a.m, a.ctl.mu, a.h0};
         LbStats ls;
-        const int status = lbfgs_solve(T, R, a.A, a.lo, a.hi, b, x, g, a.v64[2], w, gw, a.S, a.Y, a.n, c, ls, lsm);
+        const int status = lbfgs_solve(T, R, A, a.lo, a.hi, b, x, g, a.v64[2], w, gw, a.S, a.Y, a.n, c, ls, lsm);
         if (status == ST_TIMEOUT) return;
         if (x != x0) {
             R.each([&](int64_t i) { x0[i] = x[i]; });
@@ -52,12 +69,19 @@ __global__ void __launch_bounds__(kSolveThreads) k_lbfgs_grid(GridArgs a) {
     }
 }
 
-// The same driver with the trust-region Newton solver (FP64, SELL).
-__global__ void __launch_bounds__(kSolveThreads, 2) k_tron_grid(GridArgs a) {
+// The same driver with the trust-region Newton solver (FP64, SELL).  LOCAL: the
+// block's slices of the operator in shared memory, one 512-thread block per SM
+// (mid-size systems; see the dispatch in plan_build).
+template <bool LOCAL, int TPB>
+__global__ void __launch_bounds__(TPB, LOCAL ? 1 : 2) k_tron_grid(GridArgs a) {
     __shared__ RedSmem sm;
+    extern __shared__ __align__(16) unsigned char drv_smem[];
     GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm, 0, 0};
     const Rows R = rows_of_block(a.n, a.nslices, blockIdx.x, gridDim.x);
     T.active = a.pc.ncolors > 0 ? (int)(blockDim.x >> 5) : R.active_warps(blockDim.x >> 5);
+    SellF64X<LOCAL> A;
+    if constexpr (LOCAL) A = stage_operator(a.A, R, drv_smem);
+    else A = a.A;
     double *x0 = a.v64[0];
     R.each([&](int64_t i) { x0[i] = a.c_in[a.free_node[i]]; });
     if (!T.sync()) return;
@@ -79,7 +103,7 @@ __global__ void __launch_bounds__(kSolveThreads, 2) k_tron_grid(GridArgs a) {
                    a.v64[10], b, a.dinv64, a.fmask, a.pc.ncolors > 0 ? &pcv : nullptr};
         const TronCtl c{a.rtol * den, 0.5 * a.rtol * den, a.ksp_rtol, a.ctl.max_spmv, 50};
         TronStats ts;
-        const int status = tron_solve(T, R, a.A, B, v, c, ts);
+        const int status = tron_solve(T, R, A, B, v, c, ts);
         if (status == ST_TIMEOUT) return;
         if (v.x != x0) {
             const double *xs = v.x;
@@ -489,7 +513,7 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
         a.A32.stream = true;
     }
     if (const char *e = getenv("NNQP_GRID_THREADS")) tpb = atoi(e);
-    GridKernel kern = lbfgs ? k_lbfgs_grid : tron ? k_tron_grid : grid_kernel(mode, fmt, a.ctl.cg_variant, tpb);
+    GridKernel kern = lbfgs ? k_lbfgs_grid<false> : tron ? k_tron_grid<false, kSolveThreads> : grid_kernel(mode, fmt, a.ctl.cg_variant, tpb);
     // a launch shape built only with the streamed FP32 operator: that kernel
     // stands in for the sizing below and must be taken by the streaming
     // choice further down (checked there)
@@ -567,6 +591,28 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
                 a.ctl.res_warps = !resident ? 0 : rw ? std::min(atoi(rw), kResWarps) : resident_warps(deep);
                 a.res_offset = local ? (int)op : 0;
                 a.res_table = (int)table;
+            }
+        }
+        cudaGetLastError();   // a refused attribute leaves the plain kernel in use
+    }
+    // Mid-size TRON and L-BFGS solves: the operator in shared memory, one block
+    // per SM as far as there are slices.
+    if (driver && o->grid_blocks == 0 && slices <= (int64_t)4 * 8 * sms) {
+        const int w = (int)std::min<int64_t>(slices, sms);
+        const size_t op = (size_t)((slices + w - 1) / w) * s->max_slice_slots * 12;
+        GridKernel kt = tron ? k_tron_grid<true, 512> : k_lbfgs_grid<true>;
+        const int t = tron ? 512 : kLbfgsThreads;
+        if (op > 0 && op <= kSmemOperatorBytes &&
+            cudaFuncSetAttribute((const void *)kt, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kSmemOperatorBytes) == cudaSuccess) {
+            int per = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kt, t, op);
+            if (per * sms >= w) {
+                kern = kt;
+                tpb = t;
+                dyn_smem = op;
+                maxg = per * sms;
+                want = w;
             }
         }
         cudaGetLastError();   // a refused attribute leaves the plain kernel in use

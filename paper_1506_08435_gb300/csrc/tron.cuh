@@ -236,7 +236,9 @@ __device__ int tron_solve(Team &T, const Rows &R, const Op &A, const Bounds<doub
                         const bool curv = pq > 0.0;
                         const bool out = curv && ssc + al * (2.0 * sp + al * pp) >= dd;
                         // step to the boundary: the root tau >= 0 of |s + tau p|^2 = Delta^2
-                        const double tau = (-sp + sqrt(fmax(sp * sp + pp * (dd - ssc), 0.0))) / pp;
+                        // (only then: its root and division take as long as the rest)
+                        double tau = 0.0;
+                        if (out) tau = (-sp + sqrt(fmax(sp * sp + pp * (dd - ssc), 0.0))) / pp;
                         r[0] = curv ? 1.0 : 0.0;
                         r[1] = out ? 1.0 : 0.0;
                         r[2] = al;
@@ -289,11 +291,18 @@ __device__ int tron_solve(Team &T, const Rows &R, const Op &A, const Bounds<doub
                     st.vec += 8;
                     st.fl += 11;
                 }
-                if (!team_sum(T, a2, d2)) return ST_TIMEOUT;
+                // stop test and beta, once per block by warp 0 (a division by every warp
+                // holds the FP64 units for 3,000 cycles)
+                double o2[2];
+                if (!team_sum_scalar(T, a2, d2, o2, [&](const double (&s)[3], double (&r)[2]) {
+                        r[0] = (s[1] <= ktol2 || !(s[0] > 0.0)) ? 1.0 : 0.0;
+                        r[1] = s[0] / rzc;
+                    }))
+                    return ST_TIMEOUT;
                 ++st.cg;
                 ss = d2[2];
-                if (d2[1] <= ktol2 || !(d2[0] > 0.0) || st.spmv >= C.max_spmv) break;
-                const double beta = d2[0] / rz;
+                if (flag_set(o2[0]) || st.spmv >= C.max_spmv) break;
+                const double beta = o2[1];
                 rz = d2[0];
                 R.each([&](int64_t i) { v.p[i] = v.z[i] + beta * v.p[i]; });
                 st.vec += 3;
