@@ -751,8 +751,8 @@ nn_status assemble_impl(const nn_problem *p, const nn_assemble_opts *o, cudaStre
     } while (0)
 
     int *d_status;
-    TRYF(T.a.alloc(&d_status, 1, st));
-    CUF(cudaMemsetAsync(d_status, 0, sizeof(int), st));
+    TRYF(T.a.alloc(&d_status, 4, st));   // the status word; the widest SELL slice (8 bytes, at 2)
+    CUF(cudaMemsetAsync(d_status, 0, 4 * sizeof(int), st));
 
     // ---- mesh
     TRYF(s->arena.alloc(&s->coords, (size_t)N * dim, st));
@@ -882,12 +882,8 @@ nn_status assemble_impl(const nn_problem *p, const nn_assemble_opts *o, cudaStre
     TRYF(T.a.alloc(&wslots, nslices, st));
     int64_t *sptr;
     TRYF(s->arena.alloc(&sptr, nslices + 1, st));
-    // two norms and the widest slice, read back together at the end
-    double *dn;
-    TRYF(T.a.alloc(&dn, 3 + 1024, st));
-    CUF(cudaMemsetAsync(dn, 0, 3 * sizeof(double), st));
-    (k_slice_width<<<nblk(nslices), TPB, 0, st>>>(NF, nslices, offcnt, wslots,
-                                                  reinterpret_cast<unsigned long long *>(dn + 2)), ::nnqp::count_launch());
+    unsigned long long *widest = reinterpret_cast<unsigned long long *>(d_status + 2);
+    (k_slice_width<<<nblk(nslices), TPB, 0, st>>>(NF, nslices, offcnt, wslots, widest), ::nnqp::count_launch());
     int64_t *scratch3;
     TRYF(T.a.alloc(&scratch3, scan_tmp_elems(nslices + 1) + 64, st));
     CUF(exclusive_scan(wslots, sptr, nslices, scratch3, st));
@@ -924,12 +920,16 @@ nn_status assemble_impl(const nn_problem *p, const nn_assemble_opts *o, cudaStre
                                                      transient ? s->M64.val : nullptr, s->rsum32, s->dinv32,
                                                      s->dinv64, s->diag64), ::nnqp::count_launch());
     // ---- norms
-    CUF(det_max(rabs, NF, dn, dn + 3, st));
-    CUF(det_sumsq(s->b0, NF, dn + 1, dn + 3, st));
-    double hn[3];
-    CUF(cudaMemcpyAsync(hn, dn, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    double *dn;
+    TRYF(T.a.alloc(&dn, 2 + 1024, st));
+    CUF(det_max(rabs, NF, dn, dn + 2, st));
+    CUF(det_sumsq(s->b0, NF, dn + 1, dn + 2, st));
+    double hn[2];
+    unsigned long long hw = 0;
+    CUF(cudaMemcpyAsync(hn, dn, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CUF(cudaMemcpyAsync(&hw, widest, sizeof(hw), cudaMemcpyDeviceToHost, st));
     CUF(cudaStreamSynchronize(st));
-    std::memcpy(&s->max_slice_slots, &hn[2], sizeof(int64_t));
+    s->max_slice_slots = (int64_t)hw;
     s->anorm_inf = hn[0];
     s->b0norm = std::sqrt(hn[1]);
     s->has_csr = true;  // the reduced CSR is always kept (small next to SELL; used by nn_spmv)

@@ -65,8 +65,25 @@ __device__ __forceinline__ void named_arrive(int id, int threads) {
 // alone and the block's barriers would no longer match.
 __device__ __forceinline__ bool resident_done(const RedSmem &sm, int it, int64_t left) {
     const double *sc = sm.sc + 8 * (it & 1);
-    return flag_set(sc[0]) || flag_set(sc[4]) || !flag_set(sc[3]) || sm.flag2[it & 1] == 0 || it >= left;
+    return flag_set(sc[0]) || flag_set(sc[4]) || !flag_set(sc[3]) || flag_set(sc[7]) || sm.flag2[it & 1] == 0 ||
+           it >= left;
 }
+
+// Whether it ended on the trust region's boundary (and for no other reason).
+__device__ __forceinline__ bool resident_hit(const double *sc, int it, int64_t left) {
+    return flag_set(sc[7]) && !flag_set(sc[0]) && !flag_set(sc[4]) && flag_set(sc[3]) && it < left;
+}
+
+// The trust region of TRON's subspace steps (tron.cuh; TR below).  The step ends
+// where ||s|| would reach Delta.  ||s + alpha p||, with p the next direction, is
+// followed by recurrences of s's, s'p and p'p from three more sums (u'u, u'p,
+// u's), so the test needs no pass of its own.
+struct ResidentTrust {
+    double dd;           // Delta^2
+    double ksp2, face2;  // stop at ||r||^2 <= max(ksp2 ||r_0||^2, face2), ...
+    double ktol2;        // ... set here on the phase's first step (< 0 on entry), kept for the others
+    bool hit;            // out: the step ends on the boundary
+};
 
 // Products y = A x of the rows of a compute warp's slices (local slices warp,
 // warp + na, ... < ns).  The warp issues in order and 8 multiply-adds hold the
@@ -132,11 +149,13 @@ __device__ __forceinline__ void resident_product(const Op &A, const int *sl, boo
 // One CG phase from v.x, v.g; leaves the step in v.s.  Every thread of every
 // block calls it; na compute warps.  Returns 0, ST_TIMEOUT when a wait gave
 // up, or 1 when the face has nothing to reduce.  A call of its own: the
-// registers the caller keeps live are saved once per phase.
-template <class Team, class Op, typename V>
+// registers the caller keeps live are saved once per phase.  TR: tr is its trust
+// region and the stall test is left out.
+template <bool TR, class Team, class Op, typename V>
 __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, const Bounds<V> &B,
                                         const GpcgVecs<V> &v_, const GpcgCtl &C_, GpcgStats &st, double ftol2,
-                                        int na) {
+                                        int na, ResidentTrust *tr) {
+    constexpr int K = TR ? 6 : 3;   // sums of an update: gamma, delta, r'r (, u'u, u'p, u's)
     Team T = T_;
     const Rows R = R_;
     Op A = A_;
@@ -189,7 +208,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
     bool wide = false;
     for (int t = threadIdx.x; t < ns; t += blockDim.x) wide = wide || sl[t + 1] - sl[t] > 8 * 32;
     wide = __syncthreads_or(wide);
-    Acc<V> a3[2];
+    Acc<V> a3[TR ? 4 : 2];
     if (compute)
         resident_product(
             A, sl, wide, warp, na, ns, lane, mn - base, [&](int l) { return u[l]; },
@@ -199,16 +218,52 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
                 if (l < n) mc[l] = dl * wl;
                 a3[0] += r[l] * u[l];
                 a3[1] += wl * u[l];
+                if constexpr (TR) {
+                    a3[2] += r[l] * r[l];
+                    a3[3] += u[l] * u[l];
+                }
             });
-    double d3[2], o3[7];
-    if (!team_sum_scalar(T, a3, d3, o3, [&](const double (&d)[2], double (&o)[7]) { cg_scalar_start(d, o); }))
+    double d3[TR ? 4 : 2], oc[TR ? 10 : 7], o3[7];
+    // TR: (.., outside Delta, step to it, ktol2) of the first direction u
+    if (!team_sum_scalar(T, a3, d3, oc, [&](const double (&d)[TR ? 4 : 2], double (&o)[TR ? 10 : 7]) {
+            const double d2[2] = {d[0], d[1]};
+            double o2[7];
+            cg_scalar_start(d2, o2);
+#pragma unroll
+            for (int k = 0; k < 7; ++k) o[k] = o2[k];
+            if constexpr (TR) {
+                const double kt = tr->ktol2 < 0.0 ? fmax(tr->ksp2 * d[2], tr->face2) : tr->ktol2;
+                if (tr->ktol2 >= 0.0 && d[2] <= kt) o[0] = 1.0;   // the face gradient is small enough
+                const bool out = o2[1] * o2[1] * d[3] >= tr->dd;
+                o[7] = out ? 1.0 : 0.0;
+                o[8] = out ? sqrt(tr->dd / d[3]) : 0.0;
+                o[9] = kt;
+            }
+        }))
         return ST_TIMEOUT;
     ++st.spmv;
     st.fl += 6;
+#pragma unroll
+    for (int k = 0; k < 7; ++k) o3[k] = oc[k];
+    if constexpr (TR) {
+        if (tr->ktol2 < 0.0) tr->ktol2 = oc[9];
+        ftol2 = oc[9];
+    }
     if (flag_set(o3[0])) {
         __syncthreads();
         T_ = T;
         return 1;   // no step on this face
+    }
+    if constexpr (TR) {
+        if (flag_set(oc[7])) {
+            if (compute)
+#pragma unroll 1
+                for (int l = 32 * warp + lane; l < n; l += 32 * na) v.s[base + l] = oc[8] * u[l];
+            tr->hit = true;
+            __syncthreads();
+            T_ = T;
+            return 0;
+        }
     }
     CgScalars cs;
     cg_take(cs, o3);
@@ -243,24 +298,30 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
             }
             __syncwarp();
             named_arrive(1, n1);
-            Acc<V> a4[3];   // gamma, delta, r'r
+            Acc<V> a4[K];
 #pragma unroll 1
             for (int l = 32 * warp + lane; l < nl; l += 32 * na) {
                 const V ql = y[l] + vb * q[l], pl = u[l] + vb * p[l];
                 const V rl = r[l] - va * ql, ul = di[l] * rl;
                 q[l] = ql;
                 p[l] = pl;
-                s[l] = s[l] + va * pl;
+                const V sn = s[l] + va * pl;
+                s[l] = sn;
                 r[l] = rl;
                 u[l] = ul;
                 a4[0] += rl * ul;
                 a4[1] += w[l] * ul;
                 a4[2] += rl * rl;
+                if constexpr (TR) {
+                    a4[3] += ul * ul;
+                    a4[4] += ul * pl;
+                    a4[5] += ul * sn;
+                }
             }
-            double d4[3];
+            double d4[K];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) d4[k] = a4[k].value();
-            warp_stage<3>(d4, sm);
+            for (int k = 0; k < K; ++k) d4[k] = a4[k].value();
+            warp_stage<K>(d4, sm);
             __syncwarp();
             named_arrive(3, n1);
             ++it;
@@ -269,8 +330,12 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
             mn = t;
             named_sync(2, n1);
         }
+        const double *sc = sm.sc + 8 * (it & 1);
+        const bool hit = TR && resident_hit(sc, it, left);
+        const V tau = hit ? (V)sc[6] : zero, bh = hit ? (V)sc[2] : zero;
 #pragma unroll 1
-        for (int l = 32 * warp + lane; l < n; l += 32 * na) v.s[base + l] = s[l];
+        for (int l = 32 * warp + lane; l < n; l += 32 * na)
+            v.s[base + l] = hit ? s[l] + tau * (u[l] + bh * p[l]) : s[l];
     } else if (warp == kResWarps) {
         // m of every block visible
         for (;;) {
@@ -284,7 +349,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
             if (resident_done(sm, it, left)) break;
         }
     } else if (warp > kResWarps) {
-        // sums over the block, then over the grid (entry k by warp 13 + k); then
+        // sums over the block, then over the grid (entries k, k + 3 by warp 13 + k); then
         // the scalar step of cg_scalar_step, its two divisions and the stop test
         // on a warp (and sub-core) each: warp 13 alpha, 14 beta and 1 / gamma,
         // 15 the test.  (One warp after the other it took 1,850 cycles.)
@@ -292,29 +357,49 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
         double t = cs.igamma * cs.ialpha;                          // warp 13
         double ig = cs.igamma;                                     // warp 14
         double dec = 0.5 * cs.alpha * cs.gamma, maxdec = dec;      // warp 15
+        // TR, warp 13: p'p and s'p of the update to come, s's before it
+        double pp = TR ? d3[TR ? 3 : 0] : 0.0, sp = 0.0, ss = 0.0, al = cs.alpha;
         for (;;) {
             ++it;
             double *sc = sm.sc + 8 * (it & 1);
             if (k == 0) {
                 named_sync(3, n1);
-                warp0_sum_warps<3>(sm, na);
+                warp0_sum_warps<K>(sm, na);
                 __syncwarp();
-                const int ok = T.res_publish(it);
+                const int ok = T.template res_publish<K>(it);
                 if (lane == 0) sm.flag = ok;
                 __syncwarp();
             }
             named_sync(5, 96);
             const double sum = sm.flag ? T.res_sum(k, it) : 0.0;
             if (lane == 0) sm.bcast[8 + k] = sum;
+            if constexpr (TR) {
+                const double more = sm.flag ? T.res_sum(k + 3, it) : 0.0;
+                if (lane == 0) sm.bcast[11 + k] = more;
+            }
             named_sync(5, 96);
             const double gamma = sm.bcast[8];
             double den = 0.0;
             if (k == 0) {
                 den = fma(-gamma * gamma, t, sm.bcast[9]);         // delta - beta gamma / alpha
                 const double an = gamma / den;
+                double out = 0.0, tau = 0.0;
+                if constexpr (TR) {
+                    ss += al * (2.0 * sp + al * pp);               // after update `it`
+                    const double bn = gamma * ig, sps = sp + al * pp;
+                    pp = sm.bcast[11] + bn * (2.0 * sm.bcast[12] + bn * pp);
+                    sp = sm.bcast[13] + bn * sps;
+                    al = an;
+                    if (ss + an * (2.0 * sp + an * pp) >= tr->dd) {
+                        out = 1.0;
+                        tau = (-sp + sqrt(fmax(sp * sp + pp * (tr->dd - ss), 0.0))) / pp;
+                    }
+                }
                 if (lane == 0) {
                     sc[1] = an;
                     sc[4] = den > 0.0 ? 0.0 : 1.0;
+                    sc[6] = tau;
+                    sc[7] = out;
                 }
             } else if (k == 1) {
                 const double bn = gamma * ig;
@@ -324,7 +409,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
                     sc[5] = ig;
                 }
             } else {
-                const bool stop = dec <= eta2 * maxdec || sum <= ftol2 || !(gamma > 0.0);
+                const bool stop = (!TR && dec <= eta2 * maxdec) || sum <= ftol2 || !(gamma > 0.0);
                 if (lane == 0) {
                     sc[0] = stop ? 1.0 : 0.0;
                     sc[3] = sm.flag ? 1.0 : 0.0;
@@ -334,7 +419,8 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
             named_sync(4, n4);
             if (resident_done(sm, it, left)) break;
             if (k == 0) {
-                t = (den * sc[5]) * sc[5];
+                ig = sc[5];
+                t = (den * ig) * ig;
             } else if (k == 2) {
                 dec = 0.5 * sc[1] * gamma;
                 maxdec = dec > maxdec ? dec : maxdec;
@@ -345,11 +431,12 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
     __syncthreads();
     it = sm.its;
     if (it < 0) return ST_TIMEOUT;
+    if constexpr (TR) tr->hit = resident_hit(sm.sc + 8 * (it & 1), it, left);
     T_ = T;
     T_.res_end(it);
     st.spmv += it + 1;
     st.cg += it;
-    st.fl += 20 * (int64_t)it;
+    st.fl += (TR ? 26 : 20) * (int64_t)it;
     return 0;
 }
 

@@ -288,9 +288,11 @@ struct GpcgStats {
     double gp2 = 0.0;
 };
 
-template <class Team, class Op, typename V>
+struct ResidentTrust;
+template <bool TR, class Team, class Op, typename V>
 __device__ __noinline__ int cg_resident(Team &T, const Rows &R, const Op &A, const Bounds<V> &B,
-                                        const GpcgVecs<V> &v, const GpcgCtl &C, GpcgStats &st, double ftol2, int na);
+                                        const GpcgVecs<V> &v, const GpcgCtl &C, GpcgStats &st, double ftol2, int na,
+                                        ResidentTrust *tr);
 
 // Runs GPCG from the iterate in v.x (projected first).  On exit v.x holds
 // the final iterate, v.g its gradient (pointers may have been swapped).
@@ -427,7 +429,7 @@ __device__ int gpcg_solve(Team &T, const Rows &R, const Op &A, const Bounds<V> &
                     const Bounds<V> b = B;
                     const GpcgVecs<V> w = v;
                     const GpcgCtl c = C;
-                    const int e = cg_resident(t, r, a, b, w, c, s, ftol2, c.res_warps);
+                    const int e = cg_resident<false>(t, r, a, b, w, c, s, ftol2, c.res_warps, nullptr);
                     T = t;
                     st = s;
                     if (e == ST_TIMEOUT) return ST_TIMEOUT;

@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include "internal.h"
 #include "grid.cuh"
 #include "lbfgs.cuh"
@@ -70,17 +71,19 @@ __global__ void __launch_bounds__(kSolveThreads) k_lbfgs_grid(GridArgs a) {
 }
 
 // The same driver with the trust-region Newton solver (FP64, SELL).  LOCAL: the
-// block's slices of the operator in shared memory, one 512-thread block per SM
-// (mid-size systems; see the dispatch in plan_build).
-template <bool LOCAL, int TPB>
+// block's slices of the operator in shared memory, one 512-thread block per SM;
+// RES: the vectors of its subspace CG too (cg_resident.cuh; mid-size systems, see
+// the dispatch in plan_build).
+template <bool LOCAL, int TPB, bool RES = false>
 __global__ void __launch_bounds__(TPB, LOCAL ? 1 : 2) k_tron_grid(GridArgs a) {
     __shared__ RedSmem sm;
     extern __shared__ __align__(16) unsigned char drv_smem[];
     GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm, 0, 0};
     const Rows R = rows_of_block(a.n, a.nslices, blockIdx.x, gridDim.x);
     T.active = a.pc.ncolors > 0 ? (int)(blockDim.x >> 5) : R.active_warps(blockDim.x >> 5);
-    SellF64X<LOCAL> A;
-    if constexpr (LOCAL) A = stage_operator(a.A, R, drv_smem);
+    static_assert(!RES || LOCAL, "the resident kernel has its operator in shared memory");
+    std::conditional_t<RES, SellF64ResX<LOCAL>, SellF64X<LOCAL>> A;
+    if constexpr (LOCAL) static_cast<SellF64Local &>(A) = stage_operator(a.A, R, drv_smem);
     else A = a.A;
     double *x0 = a.v64[0];
     R.each([&](int64_t i) { x0[i] = a.c_in[a.free_node[i]]; });
@@ -100,8 +103,11 @@ __global__ void __launch_bounds__(TPB, LOCAL ? 1 : 2) k_tron_grid(GridArgs a) {
         if (!(den > 0.0)) den = a.den_fallback;
         const SsorF64 pcv = a.pc;
         TronVecs v{x0, a.v64[1], a.v64[7], a.v64[8], a.v64[2], a.v64[3], a.v64[4], a.v64[5], a.v64[6],
-                   a.v64[10], b, a.dinv64, a.fmask, a.pc.ncolors > 0 ? &pcv : nullptr};
-        const TronCtl c{a.rtol * den, 0.5 * a.rtol * den, a.ksp_rtol, a.ctl.max_spmv, 50};
+                   a.v64[10], b, a.dinv64, a.fmask, a.pc.ncolors > 0 ? &pcv : nullptr,
+                   reinterpret_cast<double *>(drv_smem + a.res_offset + a.res_table),
+                   reinterpret_cast<int *>(drv_smem + a.res_offset)};
+        const TronCtl c{a.rtol * den, 0.5 * a.rtol * den, a.ksp_rtol, a.ctl.max_spmv, 50,
+                        RES ? a.ctl.res_warps : 0};
         TronStats ts;
         const int status = tron_solve(T, R, A, B, v, c, ts);
         if (status == ST_TIMEOUT) return;
@@ -599,18 +605,26 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     // per SM as far as there are slices.
     if (driver && o->grid_blocks == 0 && slices <= (int64_t)4 * 8 * sms) {
         const int w = (int)std::min<int64_t>(slices, sms);
-        const size_t op = (size_t)((slices + w - 1) / w) * s->max_slice_slots * 12;
-        GridKernel kt = tron ? k_tron_grid<true, 512> : k_lbfgs_grid<true>;
+        const int64_t deep = (slices + w - 1) / w;
+        const size_t op = (size_t)deep * s->max_slice_slots * 12, table = ((size_t)(deep + 1) * 4 + 15) / 16 * 16;
+        const size_t both = op + table + (size_t)kResVectors * deep * 32 * 8;
+        const char *rw = getenv("NNQP_RES_WARPS");
+        const bool res = tron && !ssor && both <= kSmemBytes && !(rw && atoi(rw) < 1);
+        const size_t bytes = res ? both : op;
+        GridKernel kt = res ? k_tron_grid<true, 512, true> : tron ? k_tron_grid<true, 512> : k_lbfgs_grid<true>;
         const int t = tron ? 512 : kLbfgsThreads;
         if (op > 0 && op <= kSmemOperatorBytes &&
             cudaFuncSetAttribute((const void *)kt, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemOperatorBytes) == cudaSuccess) {
+                                 (int)(res ? kSmemBytes : kSmemOperatorBytes)) == cudaSuccess) {
             int per = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kt, t, op);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kt, t, bytes);
             if (per * sms >= w) {
                 kern = kt;
                 tpb = t;
-                dyn_smem = op;
+                dyn_smem = bytes;
+                a.ctl.res_warps = res ? resident_warps(deep) : 0;
+                a.res_offset = (int)op;
+                a.res_table = (int)table;
                 maxg = per * sms;
                 want = w;
             }

@@ -298,10 +298,11 @@ struct GridTeam {
         if ((threadIdx.x & 31) == 0) ok = arrive_and_wait_on(&bar->count2, wait2 + it);
         return __shfl_sync(0xffffffffu, ok, 0);
     }
-    // the block's three sums (sm->bcast) published, everybody's there:
+    // the block's K sums (sm->bcast) published, everybody's there:
+    template <int K>
     __device__ int res_publish(int it) {
         const int lane = threadIdx.x & 31;
-        if (lane < 3) res_partials(it)[(size_t)lane * nblocks + blockIdx.x] = sm->bcast[lane];
+        if (lane < K) res_partials(it)[(size_t)lane * nblocks + blockIdx.x] = sm->bcast[lane];
         __syncwarp();
         int ok = 1;
         if (lane == 0) ok = arrive_and_wait_on(&bar->count, wait_id + it);
@@ -447,7 +448,9 @@ struct ClusterTeam {
         __syncwarp();
         return __all_sync(0xffffffffu, wait_cluster(b, ((e - 1) >> 1) & 1));
     }
+    template <int K>
     __device__ int res_publish(int it) {
+        static_assert(K == 3, "the exchange buffers hold three sums");
         const unsigned e = (unsigned)(events + it), lane = threadIdx.x & 31;
         uint64_t *b = mb + 2 + (e & 1);
         if (lane == 0)

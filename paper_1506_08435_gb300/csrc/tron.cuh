@@ -36,6 +36,7 @@ struct TronCtl {
     double ksp_rtol;   // subspace steps stop at ||g_F|| <= ksp_rtol ||g_F(Cauchy point)||
     int64_t max_spmv;  // cap on products for this call
     int max_minor;     // subspace steps per outer iteration
+    int res_warps;     // compute warps of the resident subspace CG (cg_resident.cuh), 0 = the one below
 };
 
 struct TronStats {
@@ -52,6 +53,8 @@ struct TronVecs {
     const double *b, *dinv;
     uint8_t *fm;              // face mask of the subspace step (1 = free)
     const SsorF64 *pc;        // SSOR ordering, or nullptr for Jacobi
+    double *res;              // shared memory of the resident subspace CG
+    int *res_sl;
 };
 
 constexpr double kTronMu0 = 1e-2;     // sufficient decrease
@@ -175,139 +178,175 @@ __device__ int tron_solve(Team &T, const Rows &R, const Op &A, const Bounds<doub
         for (int mi = 0; mi < C.max_minor; ++mi) {
             if (!(st.gp2 > tol2) || st.spmv >= C.max_spmv) break;
             ++st.minor;
-            double a0[2] = {0.0, 0.0}, d0[2];
-            if (v.pc) {
-                R.each([&](int64_t i) {
-                    const double xi = v.x[i];
-                    const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
-                    v.fm[i] = fr ? 1 : 0;
-                    const double ri = fr ? -v.g[i] : 0.0;
-                    v.r[i] = ri;
-                    v.s[i] = 0.0;
-                    a0[1] += ri * ri;
-                });
-                if (!T.sync()) return ST_TIMEOUT;
-                if (!ssor_apply(T, *v.pc, v.fm, v.dinv, v.r, v.w, v.z, [&](int64_t i, double zi) {
-                        v.p[i] = zi;
-                        a0[0] += v.r[i] * zi;
-                    }))
-                    return ST_TIMEOUT;
-                ++st.pc;
-                st.vec += 7;
-                st.fl += 4;
-            } else {
-                R.each([&](int64_t i) {
-                    const double xi = v.x[i];
-                    const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
-                    v.fm[i] = fr ? 1 : 0;
-                    const double ri = fr ? -v.g[i] : 0.0;
-                    const double zi = v.dinv[i] * ri;
-                    v.r[i] = ri;
-                    v.z[i] = zi;
-                    v.p[i] = zi;
-                    v.s[i] = 0.0;
-                    a0[0] += ri * zi;
-                    a0[1] += ri * ri;
-                });
-                st.vec += 8;
-                st.fl += 5;
-            }
-            if (!team_sum(T, a0, d0)) return ST_TIMEOUT;
-            double rz = d0[0];
-            if (!(rz > 0.0)) break;                // nothing to do on this face
-            if (mi == 0) ktol2 = fmax(C.ksp_rtol * C.ksp_rtol * d0[1], C.face_tol * C.face_tol);
-            else if (d0[1] <= ktol2) break;        // the face gradient is small enough
-            const double dd = delta * delta;
-            double ss = 0.0;
             bool hit = false;
-            for (;;) {
-                double a1[3] = {0.0, 0.0, 0.0}, d1[3], o1[4];
-                A.apply(R, v.p, [&](int64_t i, double ap) {
-                    const double qi = v.fm[i] ? ap : 0.0, pi = v.p[i];
-                    v.q[i] = qi;
-                    a1[0] += pi * qi;
-                    a1[1] += pi * pi;
-                    a1[2] += v.s[i] * pi;
-                });
-                const double rzc = rz, ssc = ss;
-                if (!team_sum_scalar(T, a1, d1, o1, [&](const double (&s)[3], double (&r)[4]) {
-                        const double pq = s[0], pp = s[1], sp = s[2];
-                        const double al = rzc / pq;
-                        const bool curv = pq > 0.0;
-                        const bool out = curv && ssc + al * (2.0 * sp + al * pp) >= dd;
-                        // step to the boundary: the root tau >= 0 of |s + tau p|^2 = Delta^2
-                        // (only then: its root and division take as long as the rest)
-                        double tau = 0.0;
-                        if (out) tau = (-sp + sqrt(fmax(sp * sp + pp * (dd - ssc), 0.0))) / pp;
-                        r[0] = curv ? 1.0 : 0.0;
-                        r[1] = out ? 1.0 : 0.0;
-                        r[2] = al;
-                        r[3] = tau;
-                    }))
-                    return ST_TIMEOUT;
-                ++st.spmv;
-                st.vec += 4;
-                st.fl += 6;
-                if (!flag_set(o1[0])) break;
-                if (flag_set(o1[1])) {             // truncate on the trust-region boundary
-                    const double tau = o1[3];
-                    R.each([&](int64_t i) { v.s[i] += tau * v.p[i]; });
-                    st.vec += 3;
-                    st.fl += 2;
-                    if (!T.sync()) return ST_TIMEOUT;
-                    hit = true;
-                    break;
+            if (IsResidentOp<Op>::value && C.res_warps > 0) {
+                if constexpr (IsResidentOp<Op>::value) {
+                    // its first step fixes the tolerance; w and gw are free here
+                    ResidentTrust tr{delta * delta, C.ksp_rtol * C.ksp_rtol, C.face_tol * C.face_tol,
+                                     mi == 0 ? -1.0 : ktol2, false};
+                    GpcgVecs<double> rv{};
+                    rv.x = v.x;
+                    rv.g = v.g;
+                    rv.s = v.s;
+                    rv.gw = v.gw;
+                    rv.m2 = v.w;
+                    rv.dinv = v.dinv;
+                    rv.res = v.res;
+                    rv.res_sl = v.res_sl;
+                    GpcgCtl rc{};
+                    rc.max_spmv = C.max_spmv;
+                    rc.cg_max = 1 << 30;
+                    GpcgStats rs;
+                    rs.spmv = st.spmv;
+                    Team t = T;
+                    const Rows r = R;
+                    const Op op = A;
+                    const Bounds<double> bb = B;
+                    const int e = cg_resident<true>(t, r, op, bb, rv, rc, rs, 0.0, C.res_warps, &tr);
+                    if (e == ST_TIMEOUT) return ST_TIMEOUT;
+                    T = t;
+                    st.spmv = rs.spmv;
+                    st.cg += rs.cg;
+                    st.vec += rs.vec;
+                    st.fl += rs.fl;
+                    ktol2 = tr.ktol2;
+                    hit = tr.hit;
+                    if (e != 0) break;             // nothing to do on this face
                 }
-                const double al = o1[2];
-                double a2[3] = {0.0, 0.0, 0.0}, d2[3];
+            } else {
+                double a0[2] = {0.0, 0.0}, d0[2];
                 if (v.pc) {
                     R.each([&](int64_t i) {
-                        const double si = v.s[i] + al * v.p[i];
-                        const double ri = v.r[i] - al * v.q[i];
-                        v.s[i] = si;
+                        const double xi = v.x[i];
+                        const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
+                        v.fm[i] = fr ? 1 : 0;
+                        const double ri = fr ? -v.g[i] : 0.0;
                         v.r[i] = ri;
-                        a2[1] += ri * ri;
-                        a2[2] += si * si;
+                        v.s[i] = 0.0;
+                        a0[1] += ri * ri;
                     });
                     if (!T.sync()) return ST_TIMEOUT;
-                    if (!ssor_apply(T, *v.pc, v.fm, v.dinv, v.r, v.w, v.z,
-                                    [&](int64_t i, double zi) { a2[0] += v.r[i] * zi; }))
+                    if (!ssor_apply(T, *v.pc, v.fm, v.dinv, v.r, v.w, v.z, [&](int64_t i, double zi) {
+                            v.p[i] = zi;
+                            a0[0] += v.r[i] * zi;
+                        }))
                         return ST_TIMEOUT;
                     ++st.pc;
                     st.vec += 7;
-                    st.fl += 10;
+                    st.fl += 4;
                 } else {
                     R.each([&](int64_t i) {
-                        const double si = v.s[i] + al * v.p[i];
-                        const double ri = v.r[i] - al * v.q[i];
+                        const double xi = v.x[i];
+                        const bool fr = num_lt(B.l(i), xi) && num_lt(xi, B.h(i));
+                        v.fm[i] = fr ? 1 : 0;
+                        const double ri = fr ? -v.g[i] : 0.0;
                         const double zi = v.dinv[i] * ri;
-                        v.s[i] = si;
                         v.r[i] = ri;
                         v.z[i] = zi;
-                        a2[0] += ri * zi;
-                        a2[1] += ri * ri;
-                        a2[2] += si * si;
+                        v.p[i] = zi;
+                        v.s[i] = 0.0;
+                        a0[0] += ri * zi;
+                        a0[1] += ri * ri;
                     });
                     st.vec += 8;
-                    st.fl += 11;
+                    st.fl += 5;
                 }
-                // stop test and beta, once per block by warp 0 (a division by every warp
-                // holds the FP64 units for 3,000 cycles)
-                double o2[2];
-                if (!team_sum_scalar(T, a2, d2, o2, [&](const double (&s)[3], double (&r)[2]) {
-                        r[0] = (s[1] <= ktol2 || !(s[0] > 0.0)) ? 1.0 : 0.0;
-                        r[1] = s[0] / rzc;
-                    }))
-                    return ST_TIMEOUT;
-                ++st.cg;
-                ss = d2[2];
-                if (flag_set(o2[0]) || st.spmv >= C.max_spmv) break;
-                const double beta = o2[1];
-                rz = d2[0];
-                R.each([&](int64_t i) { v.p[i] = v.z[i] + beta * v.p[i]; });
-                st.vec += 3;
-                st.fl += 2;
-                if (!T.sync()) return ST_TIMEOUT;
+                if (!team_sum(T, a0, d0)) return ST_TIMEOUT;
+                double rz = d0[0];
+                if (!(rz > 0.0)) break;                // nothing to do on this face
+                if (mi == 0) ktol2 = fmax(C.ksp_rtol * C.ksp_rtol * d0[1], C.face_tol * C.face_tol);
+                else if (d0[1] <= ktol2) break;        // the face gradient is small enough
+                const double dd = delta * delta;
+                double ss = 0.0;
+                for (;;) {
+                    double a1[3] = {0.0, 0.0, 0.0}, d1[3], o1[4];
+                    A.apply(R, v.p, [&](int64_t i, double ap) {
+                        const double qi = v.fm[i] ? ap : 0.0, pi = v.p[i];
+                        v.q[i] = qi;
+                        a1[0] += pi * qi;
+                        a1[1] += pi * pi;
+                        a1[2] += v.s[i] * pi;
+                    });
+                    const double rzc = rz, ssc = ss;
+                    if (!team_sum_scalar(T, a1, d1, o1, [&](const double (&s)[3], double (&r)[4]) {
+                            const double pq = s[0], pp = s[1], sp = s[2];
+                            const double al = rzc / pq;
+                            const bool curv = pq > 0.0;
+                            const bool out = curv && ssc + al * (2.0 * sp + al * pp) >= dd;
+                            // step to the boundary: the root tau >= 0 of |s + tau p|^2 = Delta^2
+                            // (only then: its root and division take as long as the rest)
+                            double tau = 0.0;
+                            if (out) tau = (-sp + sqrt(fmax(sp * sp + pp * (dd - ssc), 0.0))) / pp;
+                            r[0] = curv ? 1.0 : 0.0;
+                            r[1] = out ? 1.0 : 0.0;
+                            r[2] = al;
+                            r[3] = tau;
+                        }))
+                        return ST_TIMEOUT;
+                    ++st.spmv;
+                    st.vec += 4;
+                    st.fl += 6;
+                    if (!flag_set(o1[0])) break;
+                    if (flag_set(o1[1])) {             // truncate on the trust-region boundary
+                        const double tau = o1[3];
+                        R.each([&](int64_t i) { v.s[i] += tau * v.p[i]; });
+                        st.vec += 3;
+                        st.fl += 2;
+                        if (!T.sync()) return ST_TIMEOUT;
+                        hit = true;
+                        break;
+                    }
+                    const double al = o1[2];
+                    double a2[3] = {0.0, 0.0, 0.0}, d2[3];
+                    if (v.pc) {
+                        R.each([&](int64_t i) {
+                            const double si = v.s[i] + al * v.p[i];
+                            const double ri = v.r[i] - al * v.q[i];
+                            v.s[i] = si;
+                            v.r[i] = ri;
+                            a2[1] += ri * ri;
+                            a2[2] += si * si;
+                        });
+                        if (!T.sync()) return ST_TIMEOUT;
+                        if (!ssor_apply(T, *v.pc, v.fm, v.dinv, v.r, v.w, v.z,
+                                        [&](int64_t i, double zi) { a2[0] += v.r[i] * zi; }))
+                            return ST_TIMEOUT;
+                        ++st.pc;
+                        st.vec += 7;
+                        st.fl += 10;
+                    } else {
+                        R.each([&](int64_t i) {
+                            const double si = v.s[i] + al * v.p[i];
+                            const double ri = v.r[i] - al * v.q[i];
+                            const double zi = v.dinv[i] * ri;
+                            v.s[i] = si;
+                            v.r[i] = ri;
+                            v.z[i] = zi;
+                            a2[0] += ri * zi;
+                            a2[1] += ri * ri;
+                            a2[2] += si * si;
+                        });
+                        st.vec += 8;
+                        st.fl += 11;
+                    }
+                    // stop test and beta, once per block by warp 0 (a division by every warp
+                    // holds the FP64 units for 3,000 cycles)
+                    double o2[2];
+                    if (!team_sum_scalar(T, a2, d2, o2, [&](const double (&s)[3], double (&r)[2]) {
+                            r[0] = (s[1] <= ktol2 || !(s[0] > 0.0)) ? 1.0 : 0.0;
+                            r[1] = s[0] / rzc;
+                        }))
+                        return ST_TIMEOUT;
+                    ++st.cg;
+                    ss = d2[2];
+                    if (flag_set(o2[0]) || st.spmv >= C.max_spmv) break;
+                    const double beta = o2[1];
+                    rz = d2[0];
+                    R.each([&](int64_t i) { v.p[i] = v.z[i] + beta * v.p[i]; });
+                    st.vec += 3;
+                    st.fl += 2;
+                    if (!T.sync()) return ST_TIMEOUT;
+                }
             }
             // projected search along s
             double beta = 1.0;

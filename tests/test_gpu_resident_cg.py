@@ -90,3 +90,30 @@ def test_transient_layouts(prec, blocks, monkeypatch):
         assert q["bounds_ok"] and q["kkt_rel"] <= 1e-8
         prev = out[0][k]
     assert np.abs(out[0] - out[1]).max() <= 1e-6
+
+
+@pytest.mark.parametrize("case", ["square9", "square60", "cube6", "cube13", "hole", "steps"])
+@pytest.mark.parametrize("ksp", [1e-1, 1e-3])
+def test_tron_layouts(case, ksp, monkeypatch):
+    """TRON with its subspace CG resident: the oracle's KKT test, and the
+    solution of the plain kernels (which the KKT tolerance fixes to 1e-6)."""
+    spec = dict(square9=lambda: I.config1_steady_2d(n=9), square60=lambda: I.config1_steady_2d(n=60),
+                cube6=lambda: I.config3_steady_3d(n=6), cube13=lambda: I.config3_steady_3d(n=13),
+                hole=lambda: I.cube_with_hole(1), steps=lambda: I.config2_transient_3d(n=9, nsteps=3))[case]()
+    s = P.nn_assemble(P.Problem(spec, device=torch.device(DEV)))
+    opts = P.solve_opts(solver=P.NN_SOLVER_TRON, ksp_rtol=ksp)
+    out = []
+    for warps in (None, "0"):
+        if warps is not None:
+            monkeypatch.setenv("NNQP_RES_WARPS", warps)
+        c = torch.zeros(spec.n_nodes, dtype=torch.float64, device=DEV)
+        if spec.dt > 0:
+            infos = P.nn_transient(s, torch.tensor(spec.c0, device=DEV), spec.nsteps, c, None, opts)
+        else:
+            infos = [P.nn_qp_solve(s, c, opts)]
+        assert all(i["status"] == 0 and i["kkt_rel"] <= 1e-10 for i in infos)
+        out.append(c.cpu().numpy())
+    assert np.abs(out[0] - out[1]).max() <= 1e-6 * max(np.abs(out[1]).max(), 1e-300)
+    if spec.dt == 0:
+        red, b, x_ref, _ = oracle_solution(spec)
+        compare_solution(out[0][red.free], x_ref, red.A, b, spec.lo, spec.hi)
