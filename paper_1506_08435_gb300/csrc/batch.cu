@@ -313,7 +313,12 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         cudaStream_t on = st;
         if (q > 0) {
             on = sides[q - 1].st;
-            NN_CUDA_TRY(cudaStreamWaitEvent(on, ev.e0, 0));
+            // (no early return past the join below)
+            if (cudaStreamWaitEvent(on, ev.e0, 0) != cudaSuccess) {
+                set_error("nn_batch_solve: a side stream cannot wait for the caller's");
+                lr = NN_ERR_CUDA;
+                break;
+            }
         }
         lr = launch(launches[q], dnext + q, on);
     }
