@@ -17,10 +17,9 @@
 //     the dot products' own FMAs, and the tree over the block has 4-12 warps;
 //   * the two things that every block waits for are apart and hidden.  m goes
 //     out first and its barrier (warp 12; the grid's counter count2, or a
-//     cluster's mbarriers) runs while the other
-//     five recurrences and the dot products are computed; the sums and the
-//     scalar step (warps 13-15) run while the next product is
-//     computed, which needs m only.
+//     cluster's mbarriers) runs while the other five recurrences and the dot
+//     products are computed; the sums and the scalar step (warps 13-15) run
+//     while the next product is computed, which needs m only.
 // The product of the iteration after the last one is thus computed and not
 // used (one per phase; it is counted).
 //
@@ -62,9 +61,10 @@ __device__ __forceinline__ void named_arrive(int id, int threads) {
 // Whether the phase ends after update `it`, read by every warp behind barrier
 // 4.  The words are double-buffered by the update's parity: a warp that is
 // slow to read them must not meet those of the next update, or it would leave
-// alone and the block's barriers would no longer match.
+// alone and the block's barriers would no longer match.  (They lie behind the
+// words of the phase's first reduction, which a slow warp may still read.)
 __device__ __forceinline__ bool resident_done(const RedSmem &sm, int it, int64_t left) {
-    const double *sc = sm.sc + 8 * (it & 1);
+    const double *sc = sm.sc + 16 + 8 * (it & 1);
     return flag_set(sc[0]) || flag_set(sc[4]) || !flag_set(sc[3]) || flag_set(sc[7]) || sm.flag2[it & 1] == 0 ||
            it >= left;
 }
@@ -285,8 +285,8 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
             if (it > 0) {
                 named_sync(4, n4);
                 if (resident_done(sm, it, left)) break;
-                va = (V)sm.sc[8 * (it & 1) + 1];
-                vb = (V)sm.sc[8 * (it & 1) + 2];
+                va = (V)sm.sc[16 + 8 * (it & 1) + 1];
+                vb = (V)sm.sc[16 + 8 * (it & 1) + 2];
             }
 #pragma unroll 1
             for (int l = 32 * warp + lane; l < nl; l += 32 * na) {
@@ -330,7 +330,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
             mn = t;
             named_sync(2, n1);
         }
-        const double *sc = sm.sc + 8 * (it & 1);
+        const double *sc = sm.sc + 16 + 8 * (it & 1);
         const bool hit = TR && resident_hit(sc, it, left);
         const V tau = hit ? (V)sc[6] : zero, bh = hit ? (V)sc[2] : zero;
 #pragma unroll 1
@@ -361,7 +361,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
         double pp = TR ? d3[TR ? 3 : 0] : 0.0, sp = 0.0, ss = 0.0, al = cs.alpha;
         for (;;) {
             ++it;
-            double *sc = sm.sc + 8 * (it & 1);
+            double *sc = sm.sc + 16 + 8 * (it & 1);
             if (k == 0) {
                 named_sync(3, n1);
                 warp0_sum_warps<K>(sm, na);
@@ -426,12 +426,12 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
                 maxdec = dec > maxdec ? dec : maxdec;
             }
         }
-        if (k == 0 && lane == 0) sm.its = flag_set(sm.sc[8 * (it & 1) + 3]) && sm.flag2[it & 1] ? it : -1;
+        if (k == 0 && lane == 0) sm.its = flag_set(sm.sc[16 + 8 * (it & 1) + 3]) && sm.flag2[it & 1] ? it : -1;
     }
     __syncthreads();
     it = sm.its;
     if (it < 0) return ST_TIMEOUT;
-    if constexpr (TR) tr->hit = resident_hit(sm.sc + 8 * (it & 1), it, left);
+    if constexpr (TR) tr->hit = resident_hit(sm.sc + 16 + 8 * (it & 1), it, left);
     T_ = T;
     T_.res_end(it);
     st.spmv += it + 1;

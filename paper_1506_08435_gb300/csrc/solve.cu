@@ -491,13 +491,13 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     // blocks measure alike there).  Served solves (force_tpb) do without: blocks
     // of several requests share an SM, which its shared memory would not allow,
     // and what a request returns stays the same bits.
-    // Between those and 2^20 unknowns the best form and block depend on how
-    // much of an SM's time is FP64 and how much barrier (steady solves, us per
-    // product, form 2 x 3 blocks of 256 / form 1 x 512 / form 0 x 768 threads, steady FP64): 56^3
-    // 18.6 / 17.0 / 20.9, 72^3 32.4 / 27.5 / 32.1, 80^3 41.0 / 35.5 / 38.9, 96^3
-    // 65.6 / 68.2 / 58.7; mixed, 768 threads with the streamed FP32 operator
-    // where it exceeds 48 MB: 56^3 18.7 / 12.7 / 17.8, 72^3 31.8 / 27.5 / 28.5,
-    // 80^3 32.0 / 29.6 / 28.1, 96^3 49.7 / 46.1 / 36.1.
+    // Between those and 2^20 unknowns the best form and block of a steady solve
+    // depend on how much of an SM's time is FP64 and how much barrier.  us per
+    // product with form 2 x 3 blocks of 256 / form 1 x 512 / form 0 x 768 threads:
+    // FP64 56^3 18.6 / 17.0 / 20.9, 72^3 32.4 / 27.5 / 32.1, 80^3 41.0 / 35.5 /
+    // 38.9, 96^3 65.6 / 68.2 / 58.7; mixed (768 threads: the streamed FP32
+    // operator, where it exceeds 48 MB) 56^3 18.7 / 12.7 / 17.8, 72^3 31.8 / 27.5 /
+    // 28.5, 80^3 32.0 / 29.6 / 28.1, 96^3 49.7 / 46.1 / 36.1.
     bool wide = false;   // one 512-thread block per SM
     if (large && !force_large && force_tpb == 0 && fmt == NN_FMT_SELL && a.ctl.cg_variant == 2 &&
         !mode_transient(mode) && !getenv("NNQP_CG_VARIANT")) {

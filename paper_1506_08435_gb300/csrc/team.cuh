@@ -58,7 +58,7 @@ __device__ __forceinline__ int ld_relaxed_i32(const int *p) {
 struct RedSmem {
     double warp[kMaxWarps][kMaxRed];
     double bcast[kMaxRed];
-    double sc[16];                // results of scalar steps done by warp 0
+    double sc[32];                // results of scalar steps (0-15: warp 0's; 16-31: the resident CG phase's)
     int flag;
     int flag2[2];                 // the vector barrier passed, by parity (resident CG phase)
     int its;                      // updates of the resident CG phase, -1 = a wait gave up
