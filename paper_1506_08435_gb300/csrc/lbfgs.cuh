@@ -205,23 +205,38 @@ __device__ int lbfgs_solve(Team &T, const Rows &R, const Op &A, double lo, doubl
         // ---- memory update; uv follows the pairs to their new positions
         if (flag_set(o[2])) {
             const int drop = k == m ? 1 : 0;
-            if (threadIdx.x == 0) {
-                // new dots indexed by the old positions j; after a drop old j maps to j - 1
-                if (drop)
-                    for (int i = 0; i + 1 < k; ++i)
-                        for (int j = 0; j + 1 < k; ++j) {
-                            sm.SY[i * kLbfgsMax + j] = sm.SY[(i + 1) * kLbfgsMax + j + 1];
-                            sm.YY[i * kLbfgsMax + j] = sm.YY[(i + 1) * kLbfgsMax + j + 1];
-                        }
-                const int kn = k - drop;   // old pairs kept
-                for (int j = 0; j < kn; ++j) {
-                    const int oj = j + drop;
-                    sm.SY[kn * kLbfgsMax + j] = a[LB_X + oj];
-                    sm.SY[j * kLbfgsMax + kn] = a[LB_X + kLbMaxM + oj];
-                    sm.YY[kn * kLbfgsMax + j] = sm.YY[j * kLbfgsMax + kn] = a[LB_X + 2 * kLbMaxM + oj];
+            if (threadIdx.x < 32) {
+                // new dots indexed by the old positions j; after a drop old j maps to
+                // j - 1.  A lane per entry of the kept block, then a lane per kept pair
+                // (one thread took some 2,500 cycles of shared-memory latency).
+                static_assert((kLbMaxM - 1) * (kLbMaxM - 1) <= 32, "a lane per kept entry");
+                const int l = threadIdx.x, kn = k - drop;   // kn: old pairs kept
+                if (drop) {
+                    const bool in = kn > 0 && l < kn * kn;
+                    const int i = in ? l / kn : 0, j = in ? l - i * kn : 0;
+                    double sy = 0.0, yy = 0.0;
+                    if (in) {
+                        sy = sm.SY[(i + 1) * kLbfgsMax + j + 1];
+                        yy = sm.YY[(i + 1) * kLbfgsMax + j + 1];
+                    }
+                    __syncwarp();
+                    if (in) {
+                        sm.SY[i * kLbfgsMax + j] = sy;
+                        sm.YY[i * kLbfgsMax + j] = yy;
+                    }
+                    __syncwarp();
                 }
-                sm.SY[kn * kLbfgsMax + kn] = a[LB_SY];
-                sm.YY[kn * kLbfgsMax + kn] = a[LB_YY];
+#pragma unroll
+                for (int oj = 0; oj < kLbMaxM; ++oj)
+                    if (oj >= drop && oj < k && l == oj - drop) {
+                        sm.SY[kn * kLbfgsMax + l] = a[LB_X + oj];
+                        sm.SY[l * kLbfgsMax + kn] = a[LB_X + kLbMaxM + oj];
+                        sm.YY[kn * kLbfgsMax + l] = sm.YY[l * kLbfgsMax + kn] = a[LB_X + 2 * kLbMaxM + oj];
+                    }
+                if (l == 0) {
+                    sm.SY[kn * kLbfgsMax + kn] = a[LB_SY];
+                    sm.YY[kn * kLbfgsMax + kn] = a[LB_YY];
+                }
             }
             __syncthreads();
             const int kn = k - drop;
