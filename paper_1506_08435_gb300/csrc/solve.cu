@@ -411,6 +411,7 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     const bool late = mode_transient(mode) || (force_tpb != 0 && s->dim == 3);
     a.ctl.eta1 = late ? kEta1Warm : kEta1;
     a.ctl.eta2 = late ? kEta2Warm : kEta2;
+    a.ctl.from_afar = !late;
     a.ctl.mu = 1e-4;
     // CG form: the pipelined one (one barrier per iteration) where barrier
     // latency bounds the solve; the textbook one on large systems, where the
