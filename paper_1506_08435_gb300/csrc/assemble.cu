@@ -26,6 +26,11 @@ namespace nnqp {
 
 constexpr int kMaxCand = 256;   // element-vertex incidences gathered per row
 constexpr int kMaxRow = 64;     // nonzeros per row of the node graph
+// Slices of a system up to which the host keeps the slice table (64 KB; the
+// copy replaces that of its last word).  Larger systems' blocks are sized by
+// the widest slice: their operator is not in shared memory but on 2D meshes,
+// whose slices are alike.
+constexpr int64_t kHostSlices = 8192;
 constexpr int TPB = 256;
 
 __device__ __forceinline__ void set_status(int *st, int code) { atomicCAS(st, 0, code); }
@@ -887,8 +892,17 @@ nn_status assemble_impl(const nn_problem *p, const nn_assemble_opts *o, cudaStre
     int64_t *scratch3;
     TRYF(T.a.alloc(&scratch3, scan_tmp_elems(nslices + 1) + 64, st));
     CUF(exclusive_scan(wslots, sptr, nslices, scratch3, st));
+    // Plans size a block's shared memory by its slices: a host copy, made here so
+    // that solves only read the system (threads may share it).
     int64_t stored = 0;
-    TRYF(read_scalar(sptr + nslices, &stored, st));
+    if (nslices <= kHostSlices) {
+        s->sptr_host.resize((size_t)nslices + 1);
+        CUF(cudaMemcpyAsync(s->sptr_host.data(), sptr, sizeof(int64_t) * (nslices + 1), cudaMemcpyDeviceToHost, st));
+        CUF(cudaStreamSynchronize(st));
+        stored = s->sptr_host.back();
+    } else {
+        TRYF(read_scalar(sptr + nslices, &stored, st));
+    }
     s->A64.n = NF;
     s->A64.nslices = nslices;
     s->A64.stored = stored;

@@ -328,11 +328,23 @@ void fill_info(const nn_system *s, const int64_t *cnt, const double *sc, int pre
     (void)precision;
 }
 
+// Entries of the SELL operator that a block of a grid of `blocks` holds at most.
+int64_t block_entries(const nn_system *s, int blocks) {
+    const int64_t slices = s->A64.nslices;
+    if (s->sptr_host.empty()) return (slices + blocks - 1) / blocks * s->max_slice_slots;
+    int64_t most = 0;
+    for (int b = 0; b < blocks; ++b) {
+        const Rows r = rows_of_block(s->NF, slices, b, blocks);
+        most = std::max(most, s->sptr_host[(size_t)r.s1] - s->sptr_host[(size_t)r.s0]);
+    }
+    return most;
+}
+
 // Everything one persistent solve launch needs, built once: arguments,
 // scratch, kernel, grid and shared memory.  A plan can be launched many times
 // (stream-ordered, without host synchronisation) and its results read after.
 struct GridPlan {
-    nn_system *s = nullptr;
+    const nn_system *s = nullptr;
     nn_solve_opts o{};
     int mode = 0, nsteps = 1;
     GridArgs a{};
@@ -344,9 +356,11 @@ struct GridPlan {
 
 // Builds plan P (its scratch is allocated on stream st).  force_tpb = 256 or
 // 512 fixes the threads per block (serving decides the launch shape before
-// admission); 0 lets the size decide.
-nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps, cudaStream_t st, GridPlan &P,
+// admission); 0 lets the size decide.  Threads may build plans of one system at
+// the same time: apart from the SSOR ordering nothing of it is written.
+nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nsteps, cudaStream_t st, GridPlan &P,
                      int force_tpb = 0) {
+    const nn_system *const s = sys;
     const int64_t n = s->NF, N = s->N;
     const bool mixed = mode_mixed(mode);
     const int fmt = o->format;
@@ -371,7 +385,7 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
         set_error("the SSOR preconditioner runs in FP64 on the SELL format with GPCG or TRON");
         return NN_ERR_INVALID_ARG;
     }
-    if (ssor) NN_TRY(ssor_setup(s, st));
+    if (ssor) NN_TRY(ssor_setup(sys, st));
     P.s = s;
     P.o = *o;
     P.mode = mode;
@@ -560,19 +574,9 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     const char *sm_env = getenv("NNQP_SMEM_OP");
     const bool smem_op = !(sm_env && sm_env[0] == '0');
     if (!driver && fmt == NN_FMT_SELL && tpb == 512) {
-        if (s->sptr_host.empty()) {
-            s->sptr_host.resize((size_t)slices + 1);
-            NN_CUDA_TRY(cudaMemcpyAsync(s->sptr_host.data(), s->A64.sptr, sizeof(int64_t) * (slices + 1),
-                                        cudaMemcpyDeviceToHost, st));
-            NN_CUDA_TRY(cudaStreamSynchronize(st));
-        }
         const int vbytes = mixed ? 4 : 8;
-        int64_t most = 0;
-        for (int b = 0; b < want; ++b) {
-            const Rows rb = rows_of_block(n, slices, b, want);
-            most = std::max(most, s->sptr_host[(size_t)rb.s1] - s->sptr_host[(size_t)rb.s0]);
-        }
         const int64_t deep = (slices + want - 1) / want;   // slices of a block at most
+        const int64_t most = block_entries(s, want);
         const size_t op = (size_t)most * (4 + vbytes), table = ((size_t)(deep + 1) * 4 + 15) / 16 * 16;
         const size_t vecs = table + (size_t)kResVectors * deep * 32 * vbytes;
         const char *rw = getenv("NNQP_RES_WARPS");
@@ -639,16 +643,7 @@ nn_status plan_build(nn_system *s, const nn_solve_opts *o, int mode, int nsteps,
     const char *tma_env = getenv("NNQP_TMA_OP");
     if (!driver && fmt == NN_FMT_SELL && mixed && tpb == kLargeThreads && a.ctl.cg_variant == 0 && a.A32.stream &&
         dyn_smem == 0 && !(tma_env && tma_env[0] == '0')) {
-        if (s->sptr_host.empty()) {
-            s->sptr_host.resize((size_t)slices + 1);
-            NN_CUDA_TRY(cudaMemcpyAsync(s->sptr_host.data(), s->A64.sptr, sizeof(int64_t) * (slices + 1),
-                                        cudaMemcpyDeviceToHost, st));
-            NN_CUDA_TRY(cudaStreamSynchronize(st));
-        }
-        int64_t wmax = 0;
-        for (int64_t k = 0; k < slices; ++k)
-            wmax = std::max<int64_t>(wmax, (s->sptr_host[(size_t)k + 1] - s->sptr_host[(size_t)k]) >> 5);
-        const int se = (int)(32 * std::max<int64_t>(wmax, 2));
+        const int se = (int)std::max<int64_t>(s->max_slice_slots, 64);
         const size_t budget = kTmaSmemBytes;
         // as many slots per warp as the budget holds (2 .. 4): D - 1 slices
         // of every warp in flight
