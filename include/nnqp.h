@@ -442,7 +442,10 @@ nn_status nn_shard_spmv(int64_t nrows, const int64_t *local_rowptr, const int32_
  * 512 threads x up to 16 CTAs: each system gets a cluster of 1/2/4/8/16 CTAs by
  * its size, one launch per cluster size side by side.  c[i] is the full node vector
  * of system i (device memory).  infos: NULL or [count].  Mixed precision
- * uses FP32 inner solves with FP64 refinement per system.  Synchronizes. */
+ * uses FP32 inner solves with FP64 refinement per system.  Returns TIMEOUT if
+ * a wait within a cluster ran past wait_timeout_s (the status of the systems
+ * it was working on, and of those not begun; the others are solved).
+ * Synchronizes. */
 nn_status nn_batch_solve(int count, nn_system *const *systems, double *const *c, const nn_solve_opts *o,
                          void *stream, nn_solve_info *infos);
 

@@ -218,7 +218,9 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
     NN_CUDA_TRY(cudaMemcpyAsync(dinst, h.data(), sizeof(BatchInst) * count, cudaMemcpyHostToDevice, st));
     NN_CUDA_TRY(cudaMemcpyAsync(dorder, order.data(), sizeof(int) * count, cudaMemcpyHostToDevice, st));
     NN_CUDA_TRY(cudaMemsetAsync(dnext, 0, sizeof(unsigned) * nl, st));
-    NN_CUDA_TRY(cudaMemsetAsync(dcnt, 0, sizeof(int64_t) * count * kBatchCounters, st));
+    // (-1: an instance that no cluster took, as every one of its class gave up)
+    NN_CUDA_TRY(cudaMemsetAsync(dcnt, 0xff, sizeof(int64_t) * count * kBatchCounters, st));
+    NN_CUDA_TRY(cudaMemsetAsync(dsc, 0xff, sizeof(double) * 2 * count, st));
     GpcgCtl ctl;
     ctl.tol = 0;
     ctl.face_tol = 0;
@@ -262,28 +264,33 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         NN_CUDA_TRY(cudaStreamCreateWithFlags(&x.st, cudaStreamNonBlocking));
         NN_CUDA_TRY(cudaEventCreateWithFlags(&x.done, cudaEventDisableTiming));
     }
+    // bound on the waits of the resident kernel; NNQP_TEST_STALL_BARRIER=1 makes
+    // them run out, as in a single solve
+    const unsigned long long wait_ns = (unsigned long long)(o->wait_timeout_s * 1e9);
+    const char *stall = getenv("NNQP_TEST_STALL_BARRIER");
+    const int wait_extra = stall && stall[0] == '1' ? 1 : 0;
     // one launch of class l on stream q
     auto launch = [&](const Launch &l, unsigned *next, cudaStream_t q) -> nn_status {
         const bool res = resident_shape(shape) && l.shape.tpb == 512;
         const int C = l.shape.cluster, tpb = res ? kBatchResThreads : C > 1 ? 256 : l.shape.tpb;
-        BatchKernel k = res ? (mixed ? batch_res_kernel_mixed(l.local) : batch_res_kernel_fp64(l.local))
-                            : pick_kernel(mixed, tpb, C, ctl.cg_variant);
+        const BatchResKernel kr = !res ? nullptr : mixed ? batch_res_kernel_mixed(l.local) : batch_res_kernel_fp64(l.local);
+        BatchKernel kp = res ? nullptr : pick_kernel(mixed, tpb, C, ctl.cg_variant);
+        const void *k = res ? (const void *)kr : (const void *)kp;
         if (!k) {
             set_error("nn_batch_solve: no kernel for %d threads x %d CTAs, CG variant %d", tpb, C, ctl.cg_variant);
             return NN_ERR_INVALID_ARG;
         }
         if (!res && C <= 1) {
             int per = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, tpb, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kp, tpb, 0);
             const int grid = std::max(1, std::min(l.count, std::max(per, 1) * sms));
-            (k<<<grid, tpb, 0, q>>>(dinst, dorder + l.first, l.count, next, ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc),
+            (kp<<<grid, tpb, 0, q>>>(dinst, dorder + l.first, l.count, next, ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc),
              count_launch());
             return NN_OK;
         }
         if (res)
-            NN_CUDA_TRY(cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kBatchSmemBytes));
-        if (C > 8) NN_CUDA_TRY(cudaFuncSetAttribute((const void *)k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            NN_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmemBytes));
+        if (C > 8) NN_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -297,14 +304,17 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int nclusters = 0;
-        NN_CUDA_TRY(cudaOccupancyMaxActiveClusters(&nclusters, (const void *)k, &cfg));
+        NN_CUDA_TRY(cudaOccupancyMaxActiveClusters(&nclusters, k, &cfg));
         if (nclusters < 1) {
             set_error("nn_batch_solve: clusters of %d CTAs cannot be scheduled on this device", C);
             return NN_ERR_INVALID_ARG;
         }
         cfg.gridDim = dim3(C * std::min(l.count, nclusters));
-        NN_CUDA_TRY(cudaLaunchKernelEx(&cfg, k, (const BatchInst *)dinst, (const int *)(dorder + l.first), l.count, next,
-                                       ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc));
+        const BatchInst *di = dinst;
+        const int *ord = dorder + l.first;
+        NN_CUDA_TRY(res ? cudaLaunchKernelEx(&cfg, kr, di, ord, l.count, next, ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc,
+                                             wait_ns, wait_extra)
+                        : cudaLaunchKernelEx(&cfg, kp, di, ord, l.count, next, ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc));
         count_launch();
         return NN_OK;
     };
@@ -344,9 +354,13 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
     if (ms_out) *ms_out = ms;
     nn_status worst = NN_OK;
     for (int i = 0; i < count; ++i) {
-        const int64_t *q = &hc[(size_t)i * kBatchCounters];
+        int64_t *q = &hc[(size_t)i * kBatchCounters];
         nn_solve_info inf;
         std::memset(&inf, 0, sizeof(inf));
+        if (q[0] < 0) {
+            std::fill(q, q + kBatchCounters, 0);
+            q[0] = NN_ERR_TIMEOUT;
+        }
         inf.status = (int)q[0];
         inf.spmv64 = q[1];
         inf.spmv = q[1] + q[2];
@@ -362,9 +376,10 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         inf.bytes_algo = q[1] * bytes_spmv(s->nnzF, s->NF, 8, 8) + q[2] * bytes_spmv(s->nnzF, s->NF, 4, 4) +
                          (double)q[6] * 8.0 * s->NF + (double)q[7] * 4.0 * s->NF;
         if (infos) infos[i] = inf;
-        if (inf.status != NN_OK && worst == NN_OK) worst = (nn_status)inf.status;
+        if (inf.status != NN_OK && (worst == NN_OK || inf.status == NN_ERR_TIMEOUT)) worst = (nn_status)inf.status;
     }
     if (worst == NN_ERR_NOT_CONVERGED) set_error("some batch instances reached the iteration cap");
+    else if (worst == NN_ERR_TIMEOUT) set_error("a device-side wait of the batch gave up after %.3g s", o->wait_timeout_s);
     return worst;
 }
 

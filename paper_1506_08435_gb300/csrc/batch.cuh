@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(TPB, MIXED ? 2 : 3) k_batch_cluster(const Batc
     __shared__ double xch[2 * kMaxCluster * kMaxRed];
     __shared__ int s_q;
     const unsigned rank = cluster_rank(), size = cluster_size();
-    ClusterTeam T{&sm, xch, rank, size, 0, TPB / 32, nullptr, nullptr, 0};
+    ClusterTeam T{&sm, xch, rank, size, 0, TPB / 32, nullptr, 0};
     for (;;) {
         if (rank == 0 && threadIdx.x == 0) s_q = (int)atomicAdd(next, 1u);
         T.sync();
@@ -226,16 +226,16 @@ __global__ void __launch_bounds__(kBatchResThreads, 1) k_batch_res(const BatchIn
                                                                   const int *__restrict__ order, int count,
                                                                   unsigned *next, GpcgCtl ctl, double rtol,
                                                                   double inner_rtol, int max_ref, int64_t *counters,
-                                                                  double *scalars) {
+                                                                  double *scalars, unsigned long long wait_ns,
+                                                                  int wait_extra) {
     __shared__ RedSmem sm;
     __shared__ double xch[2 * kMaxCluster * kMaxRed];
-    __shared__ double rx[2 * 3 * kMaxCluster];
-    __shared__ uint64_t mb[4];
+    __shared__ ClusterWaits cw;
     __shared__ int s_q, s_q0;
     extern __shared__ __align__(16) unsigned char dyn[];
     const unsigned rank = cluster_rank(), size = cluster_size();
-    ClusterTeam T{&sm, xch, rank, size, 0, 1, mb, rx, 0};
-    if (threadIdx.x == 0) T.res_init();
+    ClusterTeam T{&sm, xch, rank, size, 0, 1, &cw, 0};
+    if (threadIdx.x == 0) T.res_init(wait_ns, wait_extra);
     for (;;) {
         if (rank == 0 && threadIdx.x == 0) s_q = (int)atomicAdd(next, 1u);
         T.sync();
@@ -267,12 +267,15 @@ __global__ void __launch_bounds__(kBatchResThreads, 1) k_batch_res(const BatchIn
         solve_instance<MIXED, 2, true, LOCAL>(T, R, I, id, rank, size, c, rtol, inner_rtol, max_ref, counters, scalars,
                                               dyn, at, e0);
         T.sync();
+        if (cw.gave_up) break;   // (the same on every CTA; the instances left go to other clusters or stay unsolved)
     }
     T.sync();   // no CTA leaves while another may still read its shared memory
 }
 
 using BatchKernel = void (*)(const BatchInst *, const int *, int, unsigned *, GpcgCtl, double, double, int,
                              int64_t *, double *);
+using BatchResKernel = void (*)(const BatchInst *, const int *, int, unsigned *, GpcgCtl, double, double, int,
+                                int64_t *, double *, unsigned long long, int);
 
 // Kernel for threads per block tpb (128, 256, 512; clusters use 256), CTAs per
 // instance cluster (1 = one block) and CG variant cgv (0, 1, 2); nullptr if
@@ -280,7 +283,7 @@ using BatchKernel = void (*)(const BatchInst *, const int *, int, unsigned *, Gp
 BatchKernel batch_kernel_fp64(int tpb, int cluster, int cgv);
 BatchKernel batch_kernel_mixed(int tpb, int cluster, int cgv);
 // k_batch_res, any cluster size.
-BatchKernel batch_res_kernel_fp64(bool local);
-BatchKernel batch_res_kernel_mixed(bool local);
+BatchResKernel batch_res_kernel_fp64(bool local);
+BatchResKernel batch_res_kernel_mixed(bool local);
 
 }  // namespace nnqp

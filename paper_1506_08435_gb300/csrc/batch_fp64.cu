@@ -25,6 +25,6 @@ BatchKernel batch_kernel_fp64(int tpb, int cluster, int cgv) {
     }
 }
 
-BatchKernel batch_res_kernel_fp64(bool local) { return local ? k_batch_res<0, true> : k_batch_res<0, false>; }
+BatchResKernel batch_res_kernel_fp64(bool local) { return local ? k_batch_res<0, true> : k_batch_res<0, false>; }
 
 }  // namespace nnqp

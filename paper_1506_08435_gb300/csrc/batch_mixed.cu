@@ -25,6 +25,6 @@ BatchKernel batch_kernel_mixed(int tpb, int cluster, int cgv) {
     }
 }
 
-BatchKernel batch_res_kernel_mixed(bool local) { return local ? k_batch_res<1, true> : k_batch_res<1, false>; }
+BatchResKernel batch_res_kernel_mixed(bool local) { return local ? k_batch_res<1, true> : k_batch_res<1, false>; }
 
 }  // namespace nnqp

@@ -430,7 +430,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
     }
     __syncthreads();
     it = sm.its;
-    if (it < 0) return ST_TIMEOUT;
+    if (!T.res_agree(it >= 0)) return ST_TIMEOUT;
     if constexpr (TR) tr->hit = resident_hit(sm.sc + 16 + 8 * (it & 1), it, left);
     T_ = T;
     T_.res_end(it);

@@ -311,6 +311,8 @@ struct GridTeam {
     // sum k over the blocks:
     __device__ double res_sum(int k, int it) { return sum_partials(res_partials(it) + (size_t)k * nblocks, nblocks); }
     __device__ double *res_partials(int it) { return partials + (size_t)(slot ^ (it & 1)) * kMaxRed * nblocks; }
+    // (a grid's other blocks learn of a wait that ran out from the error word)
+    __device__ bool res_agree(bool ok) { return ok; }
     // after a phase of `it` events
     __device__ void res_end(int it) {
         slot ^= it & 1;
@@ -395,6 +397,14 @@ struct GridTeam {
 
 constexpr int kMaxCluster = 16;
 
+// What a CTA of a cluster waits on in the resident CG phase, in shared memory.
+struct ClusterWaits {
+    uint64_t mb[4];                  // mbarriers: [0..1] m written, [2..3] sums
+    double rx[2 * 3 * kMaxCluster];  // sums received
+    unsigned long long wait_ns;      // bound on each wait
+    int gave_up;                     // a wait of any CTA of the cluster has run out
+};
+
 // The CTAs of one thread-block cluster (all co-scheduled by the hardware).
 // Barriers are the hardware cluster barrier.  A reduction pushes each CTA's
 // block totals into every CTA's exchange buffer (remote shared-memory
@@ -408,19 +418,21 @@ struct ClusterTeam {
     unsigned rank, size;
     int slot;
     int active;                   // warps of this CTA that own rows
-    uint64_t *mb;                 // resident CG phase: mbarriers, [0..1] m written, [2..3] sums (shared memory)
-    double *rx;                   //   sums received, [2][3][kMaxCluster]
+    ClusterWaits *cw;             // resident CG phase: what it waits on (shared memory)
     int events;                   //   events passed (each uses the mbarriers of its parity)
 
     // The resident CG phase's waits (see GridTeam).  Each event uses one of two
     // mbarriers in turn: a CTA can be one event ahead of another, never two.
+    // A wait that runs out leaves the mbarriers' phases behind: res_agree makes
+    // every CTA return ST_TIMEOUT from the same phase, and none starts another.
     __device__ static uint32_t remote(const void *p, unsigned r) {
         uint32_t a;
         asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(r));
         return a;
     }
-    __device__ static int wait_cluster(uint64_t *b, unsigned parity) {
-        for (int it = 0; it < (1 << 22); ++it) {
+    __device__ int wait_cluster(uint64_t *b, unsigned parity) const {
+        unsigned long long t0 = 0;
+        for (unsigned it = 1;; ++it) {
             unsigned done;
             asm volatile(
                 "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], "
@@ -429,19 +441,28 @@ struct ClusterTeam {
                 : "r"((uint32_t)__cvta_generic_to_shared(b)), "r"(parity)
                 : "memory");
             if (done) return 1;
+            if ((it & 7u) == 0) {
+                const unsigned long long now = global_ns();
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > cw->wait_ns) return 0;
+            }
         }
-        return 0;
     }
-    __device__ void res_init() {   // by one thread, before a cluster barrier
+    // by one thread, before a cluster barrier; extra: arrivals waited for beyond
+    // the cluster's (0; 1 only in the stall test)
+    __device__ void res_init(unsigned long long wait_ns, int extra) {
+        cw->wait_ns = wait_ns;
+        cw->gave_up = 0;
+        uint64_t *mb = cw->mb;
         for (int k = 0; k < 4; ++k)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(mb + k)),
-                         "r"(k < 2 ? size : 1u)
+                         "r"(k < 2 ? size + (unsigned)extra : 1u)
                          : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __device__ int res_vector_barrier(int it) {
         const unsigned e = (unsigned)(events + it), lane = threadIdx.x & 31;
-        uint64_t *b = mb + (e & 1);
+        uint64_t *b = cw->mb + (e & 1);
         if (lane < size)
             asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote(b, lane))
                          : "memory");
@@ -452,7 +473,7 @@ struct ClusterTeam {
     __device__ int res_publish(int it) {
         static_assert(K == 3, "the exchange buffers hold three sums");
         const unsigned e = (unsigned)(events + it), lane = threadIdx.x & 31;
-        uint64_t *b = mb + 2 + (e & 1);
+        uint64_t *b = cw->mb + 2 + (e & 1);
         if (lane == 0)
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
                              (uint32_t)__cvta_generic_to_shared(b)),
@@ -461,7 +482,7 @@ struct ClusterTeam {
         for (unsigned q = lane; q < size * 3; q += 32) {
             const unsigned r = q / 3, k = q - 3 * r;
             asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u64 [%0], %1, [%2];" ::"r"(
-                             remote(rx + ((e & 1) * 3 + k) * kMaxCluster + rank, r)),
+                             remote(cw->rx + ((e & 1) * 3 + k) * kMaxCluster + rank, r)),
                          "l"(__double_as_longlong(sm->bcast[k])), "r"(remote(b, r))
                          : "memory");
         }
@@ -470,11 +491,20 @@ struct ClusterTeam {
     }
     __device__ double res_sum(int k, int it) {
         const unsigned e = (unsigned)(events + it), lane = threadIdx.x & 31;
-        double u = lane < size ? rx[((e & 1) * 3 + k) * kMaxCluster + lane] : 0.0;
+        double u = lane < size ? cw->rx[((e & 1) * 3 + k) * kMaxCluster + lane] : 0.0;
         for (int o = (int)size >> 1; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
         return u;
     }
     __device__ void res_end(int it) { events += it; }
+    // Whether the phase went well on every CTA; all threads call it.  A CTA whose
+    // wait ran out tells all others; one that did not cannot be more than a wait
+    // of its own behind, so every CTA comes here.
+    __device__ bool res_agree(bool ok) {
+        if (!ok && threadIdx.x < size)
+            asm volatile("st.shared::cluster.s32 [%0], 1;" ::"r"(remote(&cw->gave_up, threadIdx.x)) : "memory");
+        cluster_barrier();
+        return *(volatile int *)&cw->gave_up == 0;
+    }
 
     __device__ __forceinline__ static void cluster_barrier() {
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
