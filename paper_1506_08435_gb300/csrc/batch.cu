@@ -22,7 +22,7 @@ BatchKernel pick_kernel(bool mixed, int tpb, int cluster, int cgv) {
 // Launch shape of the batch kernel: threads per block and CTAs per instance
 // (1 = one block per instance, > 1 = a cluster per instance).  512 threads with
 // more than one CTA is the resident kernel with at most that many CTAs per
-// instance: each instance gets a cluster of its own size (res_cluster).
+// instance: each instance gets a cluster of its own size (batch_place.h).
 //
 // The default is 512 x 16.  A batch of 40 instances of 20 x 20 to 120 x 120
 // cells in FP64: one 256-thread block per instance (the former default) 590 ms,
@@ -34,30 +34,6 @@ struct BatchShape {
 };
 bool resident_shape(const BatchShape &s) { return s.tpb == 512 && s.cluster > 1; }
 
-// Dynamic shared memory a CTA of the resident kernel may take (its static 22 KB
-// come on top).
-constexpr size_t kBatchSmemBytes = 204 * 1024;
-
-// Where an instance of the resident kernel runs: CTAs of its cluster (0 = it
-// does not fit: the 256-thread cluster kernel takes it) and whether its operator
-// is in shared memory.  As few CTAs as give each at most `target` slices -- an
-// iteration's barrier and sums cost the same for 1 and 28 slices a CTA -- and
-// more where that is what the operator needs to fit.
-struct ResPlace {
-    int cluster = 0;
-    bool local = false;
-};
-ResPlace res_cluster(const nn_system *s, int vbytes, int64_t target, int most) {
-    const int64_t slices = s->A64.nslices;
-    for (int c = 1; c <= most; c *= 2) {
-        const int64_t per = (slices + c - 1) / c;
-        if (per <= target && batch_res_bytes(per, s->max_slice_slots, vbytes) <= kBatchSmemBytes) return {c, true};
-    }
-    const int64_t per = (slices + most - 1) / most;
-    if (batch_res_bytes(per, s->max_slice_slots, vbytes) <= kBatchSmemBytes) return {most, true};
-    if (batch_res_bytes(per, 0, vbytes) <= kBatchSmemBytes) return {most, false};
-    return {};
-}
 BatchShape g_tuned;          // process-wide choice of the autotuner
 bool g_have_tuned = false;
 
@@ -168,10 +144,40 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         bool local = false;
         int first = 0, count = 0;
         size_t smem = 0;
+        int clusters = 0;   // that the device runs at once
     };
+    // CG form of the kernels other than the resident one
+    const char *cgv_env = getenv("NNQP_BATCH_CG_VARIANT");
+    const int cgv = cgv_env ? atoi(cgv_env) : 0;
+    // Clusters of C CTAs of kernel k that the device runs at once, 0 = none.
+    // NNQP_TEST_MAX_CLUSTER stands for a device that schedules none of more CTAs.
+    const char *mc_env = getenv("NNQP_TEST_MAX_CLUSTER");
+    const int max_cluster = mc_env ? atoi(mc_env) : kMaxCluster;
+    auto schedulable = [&](const void *k, int tpb, int C, size_t smem) {
+        if (!k || C > max_cluster) return 0;
+        int n = 0;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = C;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.blockDim = dim3(tpb);
+        cfg.gridDim = dim3(C * std::max(1, sms / C));
+        cfg.dynamicSmemBytes = smem;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if ((smem && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) ||
+            (C > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+            cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess)
+            n = 0;
+        cudaGetLastError();   // a refusal means the next choice
+        return n;
+    };
+    auto res_kernel = [&](bool local) { return mixed ? batch_res_kernel_mixed(local) : batch_res_kernel_fp64(local); };
     std::vector<Launch> launches;
     if (!resident_shape(shape)) {
-        launches.push_back({shape, false, 0, count, 0});
+        launches.push_back({shape, false, 0, count, 0, 0});
     } else {
         // slices per CTA: what spreads the whole batch over the SMs, from 4 (a
         // warp each) to 24 (three a warp).  Measured with 8 / 16 / 24 / 36: 40
@@ -182,8 +188,19 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         for (int i = 0; i < count; ++i) total += systems[i]->A64.nslices;
         const int64_t target = std::min<int64_t>(24, std::max<int64_t>(4, total / sms));
         const int vbytes = mixed ? 4 : 8;
+        // (one CTA of the resident kernel fills an SM's registers, so the count does
+        // not depend on how much of the shared memory a class takes)
+        int at_once[2][kMaxCluster + 1];
+        std::fill(&at_once[0][0], &at_once[0][0] + 2 * (kMaxCluster + 1), -1);
+        auto clusters = [&](int c, bool local) {
+            int &n = at_once[local][c];
+            if (n < 0) n = schedulable((const void *)res_kernel(local), kBatchResThreads, c, kBatchSmemBytes);
+            return n;
+        };
         std::vector<ResPlace> place(count);
-        for (int i = 0; i < count; ++i) place[i] = res_cluster(systems[i], vbytes, target, shape.cluster);
+        for (int i = 0; i < count; ++i)
+            place[i] = place_instance(systems[i]->A64.nslices, systems[i]->max_slice_slots, vbytes, target, shape.cluster,
+                                      [&](int c, bool local) { return clusters(c, local) > 0; });
         auto key = [&](int i) { return place[i].cluster == 0 ? 64 : 2 * place[i].cluster + (place[i].local ? 0 : 1); };
         std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key(a) > key(b); });
         for (int q = 0; q < count; ++q) {
@@ -191,8 +208,13 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
             const ResPlace &pl = place[i];
             if (q == 0 || key(i) != key(order[q - 1])) {
                 Launch l;
-                l.shape = pl.cluster ? BatchShape{512, pl.cluster} : BatchShape{256, 16};
+                l.shape = BatchShape{512, pl.cluster};
+                if (!pl.cluster)
+                    l.shape = {256, plain_cluster(kMaxCluster, [&](int c) {
+                                   return schedulable((const void *)pick_kernel(mixed, 256, c, cgv), 256, c, 0) > 0;
+                               })};
                 l.local = pl.local;
+                l.clusters = pl.cluster ? clusters(pl.cluster, pl.local) : 0;
                 l.first = q;
                 launches.push_back(l);
             }
@@ -231,15 +253,31 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
     ctl.eta2 = kEta2;
     ctl.from_afar = 0;   // (the batch has a cap of its own)
     ctl.mu = 1e-4;
-    ctl.cg_variant = 0;
+    ctl.cg_variant = cgv;
     ctl.cg_bound_stop = 0;
     ctl.keep_p = 0;
     ctl.res_warps = 0;
-    if (const char *e = getenv("NNQP_BATCH_CG_VARIANT")) ctl.cg_variant = atoi(e);
     if (const char *e = getenv("NNQP_CG_BOUND_STOP")) ctl.cg_bound_stop = atoi(e);
     if (const char *e = getenv("NNQP_GP_MAX")) ctl.gp_max = atoi(e);
     if (const char *e = getenv("NNQP_ETA1")) ctl.eta1 = atof(e);
     if (const char *e = getenv("NNQP_ETA2")) ctl.eta2 = atof(e);
+    // what may refuse a class comes before the first launch: a refused call has
+    // touched no c[i]
+    for (Launch &l : launches) {
+        if (resident_shape(shape) && l.shape.tpb == 512) continue;   // (as placed)
+        const int C = l.shape.cluster, tpb = C > 1 ? 256 : l.shape.tpb;
+        BatchKernel k = pick_kernel(mixed, tpb, C, cgv);
+        if (!k) {
+            set_error("nn_batch_solve: no kernel for %d threads x %d CTAs, CG variant %d", tpb, C, cgv);
+            return NN_ERR_INVALID_ARG;
+        }
+        if (C <= 1) continue;
+        l.clusters = schedulable((const void *)k, tpb, C, 0);
+        if (l.clusters < 1) {
+            set_error("nn_batch_solve: clusters of %d CTAs cannot be scheduled on this device", C);
+            return NN_ERR_INVALID_ARG;
+        }
+    }
     // The classes run side by side: the first on the caller's stream, each other
     // one on a stream of its own between two events of the caller's.
     struct Side {
@@ -273,13 +311,7 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
     auto launch = [&](const Launch &l, unsigned *next, cudaStream_t q) -> nn_status {
         const bool res = resident_shape(shape) && l.shape.tpb == 512;
         const int C = l.shape.cluster, tpb = res ? kBatchResThreads : C > 1 ? 256 : l.shape.tpb;
-        const BatchResKernel kr = !res ? nullptr : mixed ? batch_res_kernel_mixed(l.local) : batch_res_kernel_fp64(l.local);
-        BatchKernel kp = res ? nullptr : pick_kernel(mixed, tpb, C, ctl.cg_variant);
-        const void *k = res ? (const void *)kr : (const void *)kp;
-        if (!k) {
-            set_error("nn_batch_solve: no kernel for %d threads x %d CTAs, CG variant %d", tpb, C, ctl.cg_variant);
-            return NN_ERR_INVALID_ARG;
-        }
+        const BatchKernel kp = res ? nullptr : pick_kernel(mixed, tpb, C, cgv);
         if (!res && C <= 1) {
             int per = 0;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kp, tpb, 0);
@@ -288,9 +320,6 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
              count_launch());
             return NN_OK;
         }
-        if (res)
-            NN_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmemBytes));
-        if (C > 8) NN_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -298,21 +327,14 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         cfg.blockDim = dim3(tpb);
-        cfg.gridDim = dim3(C * std::max(1, sms / C));
+        cfg.gridDim = dim3(C * std::min(l.count, l.clusters));
         cfg.dynamicSmemBytes = l.smem;
         cfg.stream = q;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        int nclusters = 0;
-        NN_CUDA_TRY(cudaOccupancyMaxActiveClusters(&nclusters, k, &cfg));
-        if (nclusters < 1) {
-            set_error("nn_batch_solve: clusters of %d CTAs cannot be scheduled on this device", C);
-            return NN_ERR_INVALID_ARG;
-        }
-        cfg.gridDim = dim3(C * std::min(l.count, nclusters));
         const BatchInst *di = dinst;
         const int *ord = dorder + l.first;
-        NN_CUDA_TRY(res ? cudaLaunchKernelEx(&cfg, kr, di, ord, l.count, next, ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc,
+        NN_CUDA_TRY(res ? cudaLaunchKernelEx(&cfg, res_kernel(l.local), di, ord, l.count, next, ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc,
                                              wait_ns, wait_extra)
                         : cudaLaunchKernelEx(&cfg, kp, di, ord, l.count, next, ctl, o->rtol, o->inner_rtol, 200, dcnt, dsc));
         count_launch();

@@ -38,13 +38,6 @@ struct BatchInst {
 
 constexpr int kBatchResThreads = 512;
 
-// Shared memory of a CTA with `per` slices at most, of at most `slots` entries
-// each, `vbytes` bytes a value (0 slots: the operator stays in global memory).
-__host__ __device__ __forceinline__ size_t batch_res_table(int64_t per) { return ((size_t)(per + 1) * 4 + 15) / 16 * 16; }
-__host__ __device__ __forceinline__ size_t batch_res_bytes(int64_t per, int64_t slots, int vbytes) {
-    return (size_t)per * slots * (4 + vbytes) + batch_res_table(per) + (size_t)kResVectors * per * 32 * vbytes;
-}
-
 constexpr int kBatchCounters = 9;
 
 // Solves instance `id` with team T; this CTA owns the rows R of it.

@@ -37,11 +37,11 @@
 #include <stdint.h>
 #include "team.cuh"
 #include "ops.cuh"
+#include "batch_place.h"
 
 namespace nnqp {
 
 constexpr int kResWarps = 12;         // compute warps at most; warps 12-15 serve (512-thread blocks)
-constexpr int kResVectors = 9;        // vectors of the block's rows in shared memory
 
 // Compute warps for at most `per` slices a block: 8 (two a sub-core) up to
 // three slices a warp, then 12; 4 where a warp has one slice at most.
