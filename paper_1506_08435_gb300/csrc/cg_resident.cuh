@@ -381,7 +381,9 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
             const double gamma = sm.bcast[8];
             double den = 0.0;
             if (k == 0) {
-                den = fma(-gamma * gamma, t, sm.bcast[9]);         // delta - beta gamma / alpha
+                // delta - beta gamma / alpha (gamma t = beta / alpha first: gamma^2
+                // leaves the range where gamma, a square of the data, does not)
+                den = fma(-(gamma * t), gamma, sm.bcast[9]);
                 const double an = gamma / den;
                 double out = 0.0, tau = 0.0;
                 if constexpr (TR) {
@@ -392,7 +394,8 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
                     al = an;
                     if (ss + an * (2.0 * sp + an * pp) >= tr->dd) {
                         out = 1.0;
-                        tau = (-sp + sqrt(fmax(sp * sp + pp * (tr->dd - ss), 0.0))) / pp;
+                        const double h = sp / pp;                  // (not sp^2, for the same reason)
+                        tau = sqrt(fmax(h * h + (tr->dd - ss) / pp, 0.0)) - h;
                     }
                 }
                 if (lane == 0) {
