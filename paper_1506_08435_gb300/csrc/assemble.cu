@@ -888,7 +888,8 @@ nn_status assemble_impl(const nn_problem *p, const nn_assemble_opts *o, cudaStre
     int64_t *sptr;
     TRYF(s->arena.alloc(&sptr, nslices + 1, st));
     unsigned long long *widest = reinterpret_cast<unsigned long long *>(d_status + 2);
-    (k_slice_width<<<nblk(nslices), TPB, 0, st>>>(NF, nslices, offcnt, wslots, widest), ::nnqp::count_launch());
+    (k_slice_width<<<nblk(nslices), TPB, 0, st>>>(NF, nslices, offcnt, wslots, nslices <= kHostSlices ? nullptr : widest),
+     ::nnqp::count_launch());
     int64_t *scratch3;
     TRYF(T.a.alloc(&scratch3, scan_tmp_elems(nslices + 1) + 64, st));
     CUF(exclusive_scan(wslots, sptr, nslices, scratch3, st));
@@ -941,9 +942,11 @@ nn_status assemble_impl(const nn_problem *p, const nn_assemble_opts *o, cudaStre
     double hn[2];
     unsigned long long hw = 0;
     CUF(cudaMemcpyAsync(hn, dn, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CUF(cudaMemcpyAsync(&hw, widest, sizeof(hw), cudaMemcpyDeviceToHost, st));
+    if (s->sptr_host.empty()) CUF(cudaMemcpyAsync(&hw, widest, sizeof(hw), cudaMemcpyDeviceToHost, st));
     CUF(cudaStreamSynchronize(st));
     s->max_slice_slots = (int64_t)hw;
+    for (size_t k = 1; k < s->sptr_host.size(); ++k)
+        s->max_slice_slots = std::max(s->max_slice_slots, s->sptr_host[k] - s->sptr_host[k - 1]);
     s->anorm_inf = hn[0];
     s->b0norm = std::sqrt(hn[1]);
     s->has_csr = true;  // the reduced CSR is always kept (small next to SELL; used by nn_spmv)
