@@ -606,15 +606,18 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
         }
         cudaGetLastError();   // a refused attribute leaves the plain kernel in use
     }
-    // Mid-size TRON and L-BFGS solves: the operator in shared memory, one block
-    // per SM as far as there are slices.
-    if (driver && o->grid_blocks == 0 && slices <= (int64_t)4 * 8 * sms) {
+    // Mid-size TRON (with Jacobi) and L-BFGS solves: the operator in shared
+    // memory, one block per SM as far as there are slices.  SSOR spreads its
+    // colours over all warps of a plain grid of 256-thread blocks: 512-thread
+    // blocks with the operator in shared memory are 1 to 6% slower alone (50 x 50
+    // 16.0 -> 17.1 ms, 30^3 68.5 -> 72.2) and half as many solves a second.
+    if (driver && !ssor && o->grid_blocks == 0 && slices <= (int64_t)4 * 8 * sms) {
         const int w = (int)std::min<int64_t>(slices, sms);
         const int64_t deep = (slices + w - 1) / w;
         const size_t op = (size_t)deep * s->max_slice_slots * 12, table = ((size_t)(deep + 1) * 4 + 15) / 16 * 16;
         const size_t both = op + table + (size_t)kResVectors * deep * 32 * 8;
         const char *rw = getenv("NNQP_RES_WARPS");
-        const bool res = tron && !ssor && both <= kSmemBytes && !(rw && atoi(rw) < 1);
+        const bool res = tron && both <= kSmemBytes && !(rw && atoi(rw) < 1);
         const size_t bytes = res ? both : op;
         GridKernel kt = res ? k_tron_grid<true, 512, true> : tron ? k_tron_grid<true, 512> : k_lbfgs_grid<true>;
         const int t = tron ? 512 : kLbfgsThreads;
