@@ -16,9 +16,9 @@
 //   * few compute warps with several slices each: a thread's rows are added by
 //     the dot products' own FMAs, and the tree over the block has 4-12 warps;
 //   * the two things that every block waits for are apart and hidden.  m goes
-//     out first and its barrier (warp 12; the grid's counter count2, or a
+//     out first and its barrier (the first serving warp; the grid's counter count2, or a
 //     cluster's mbarriers) runs while the other five recurrences and the dot
-//     products are computed; the sums and the scalar step (warps 13-15) run
+//     products are computed; the sums and the scalar step (the other three) run
 //     while the next product is computed, which needs m only.
 // The product of the iteration after the last one is thus computed and not
 // used (one per phase; it is counted).
@@ -41,7 +41,10 @@
 
 namespace nnqp {
 
-constexpr int kResWarps = 12;         // compute warps at most; warps 12-15 serve (512-thread blocks)
+// Compute warps at most.  A block's last four warps serve: 12-15 of 512-thread
+// blocks; 4-7 of the 256-thread blocks of systems with at most four slices a
+// block, of which two share an SM.
+constexpr int kResWarps = 12;
 
 // Compute warps for at most `per` slices a block: 8 (two a sub-core) up to
 // three slices a warp, then 12; 4 where a warp has one slice at most.
@@ -167,6 +170,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
     const double eta2 = C_.eta2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool compute = warp < na;
+    const int serve = (int)(blockDim.x >> 5) - 4;   // the first serving warp
     RedSmem &sm = *in_shared(T.sm);
     const V zero = (V)0;
     const int ns = (int)(R.s1 - R.s0), nl = ns * 32, base = (int)(R.s0 * 32);
@@ -336,7 +340,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
 #pragma unroll 1
         for (int l = 32 * warp + lane; l < n; l += 32 * na)
             v.s[base + l] = hit ? s[l] + tau * (u[l] + bh * p[l]) : s[l];
-    } else if (warp == kResWarps) {
+    } else if (warp == serve) {
         // m of every block visible
         for (;;) {
             named_sync(1, n1);
@@ -348,16 +352,16 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
             named_sync(4, n4);
             if (resident_done(sm, it, left)) break;
         }
-    } else if (warp > kResWarps) {
-        // sums over the block, then over the grid (entries k, k + 3 by warp 13 + k); then
+    } else if (warp > serve) {
+        // sums over the block, then over the grid (entries k, k + 3 by serving warp 1 + k); then
         // the scalar step of cg_scalar_step, its two divisions and the stop test
-        // on a warp (and sub-core) each: warp 13 alpha, 14 beta and 1 / gamma,
-        // 15 the test.  (One warp after the other it took 1,850 cycles.)
-        const int k = warp - (kResWarps + 1);
-        double t = cs.igamma * cs.ialpha;                          // warp 13
-        double ig = cs.igamma;                                     // warp 14
-        double dec = 0.5 * cs.alpha * cs.gamma, maxdec = dec;      // warp 15
-        // TR, warp 13: p'p and s'p of the update to come, s's before it
+        // on a warp (and sub-core) each: k = 0 alpha, 1 beta and 1 / gamma, 2 the
+        // test.  (One warp after the other it took 1,850 cycles.)
+        const int k = warp - (serve + 1);
+        double t = cs.igamma * cs.ialpha;                          // k = 0
+        double ig = cs.igamma;                                     // k = 1
+        double dec = 0.5 * cs.alpha * cs.gamma, maxdec = dec;      // k = 2
+        // TR, k = 0: p'p and s'p of the update to come, s's before it
         double pp = TR ? d3[TR ? 3 : 0] : 0.0, sp = 0.0, ss = 0.0, al = cs.alpha;
         for (;;) {
             ++it;

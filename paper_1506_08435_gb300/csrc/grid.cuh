@@ -162,7 +162,7 @@ __device__ bool step_outputs(Team &T, const Rows &R, const GridArgs &a, const do
 // vectors in shared memory (cg_resident.cuh; kernels of their own, as its code
 // costs the plain phase registers).
 template <int FMT, int MODE, int CGV, int TPB>
-__global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k_solve_grid(GridArgs a) {
+__global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : FMT >= 4 ? 2 : mode_min_blocks(MODE)) k_solve_grid(GridArgs a) {
     __shared__ RedSmem sm;
     extern __shared__ __align__(16) unsigned char op_smem[];
     GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm, 0, 0};
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : mode_min_blocks(MODE)) k
     R.each([&](int64_t i) { x[i] = a.c_in[a.free_node[i]]; });
     // shared memory of the resident CG phase (behind the operator of FMT 2)
     constexpr bool RES = FMT == 4 || FMT == 5, LOCAL = FMT == 2 || FMT == 4;
-    static_assert(!RES || (CGV == 2 && TPB == 512), "the resident CG phase is form 2 in 512-thread blocks");
+    static_assert(!RES || (CGV == 2 && (TPB == 512 || TPB == 256)), "the resident CG phase is form 2");
     [[maybe_unused]] unsigned char *res = op_smem + a.res_offset;
     SellF64Local Aloc{};
     SellF32DiffLocal A32loc{};

@@ -71,11 +71,11 @@ __global__ void __launch_bounds__(kSolveThreads) k_lbfgs_grid(GridArgs a) {
 }
 
 // The same driver with the trust-region Newton solver (FP64, SELL).  LOCAL: the
-// block's slices of the operator in shared memory, one 512-thread block per SM;
-// RES: the vectors of its subspace CG too (cg_resident.cuh; mid-size systems, see
+// block's slices of the operator in shared memory, one 512-thread block per SM
+// (256 threads: two, small systems); RES: the vectors of its subspace CG too (cg_resident.cuh; mid-size systems, see
 // the dispatch in plan_build).
 template <bool LOCAL, int TPB, bool RES = false>
-__global__ void __launch_bounds__(TPB, LOCAL ? 1 : 2) k_tron_grid(GridArgs a) {
+__global__ void __launch_bounds__(TPB, LOCAL && TPB == 512 ? 1 : 2) k_tron_grid(GridArgs a) {
     __shared__ RedSmem sm;
     extern __shared__ __align__(16) unsigned char drv_smem[];
     GridTeam T{a.bar, a.partials, (int)gridDim.x + a.bar_extra, a.timeout_ns, 0, 0, &sm, 0, 0};
@@ -500,12 +500,16 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
     // load-based kernel where the streamed operator does not apply).
     const bool large = !driver && (slices > (int64_t)4 * 8 * sms || force_large);
     // The pipelined CG form of those systems keeps its vectors on the SM
-    // (cg_resident.cuh) in 512-thread blocks, which the smallest systems gain
-    // from as well (50 x 50: 5.3 ms in 19 blocks of 256 threads, 3.9 ms here);
-    // their slices are spread one to a block as far as there are SMs (12 to 76
-    // blocks measure alike there).  Served solves (force_tpb) do without: blocks
-    // of several requests share an SM, which its shared memory would not allow,
-    // and what a request returns stays the same bits.
+    // (cg_resident.cuh) in 512-thread blocks, one per SM.  With at most four
+    // slices per SM (`few`) four compute warps do, so the blocks have 256 threads,
+    // two fit an SM, and four slices to a block leave the other SMs to solves on
+    // other streams.  Alone / 16 host threads with a system and a stream each, in
+    // 256-thread blocks without the resident phase, one slice to a 512-thread
+    // block, and so: 50 x 50 5.45 / 4.56 / 4.20 ms and 1,400 / 540 / 2,150 solves
+    // a second, 100 x 100 12.2 / 8.5 / 8.4 ms and 171 / 107 / 275, 14^3 steps
+    // 2.10 / 1.95 / 1.85 ms and 3,250 / 530 / 3,620.  Fewer slices to a block (1
+    // to 3) are no faster alone (within 1%).  Served solves (force_tpb) do
+    // without the resident phase: their launch shapes are fixed before admission.
     // Between those and 2^20 unknowns the best form and block of a steady solve
     // depend on how much of an SM's time is FP64 and how much barrier.  us per
     // product with form 2 x 3 blocks of 256 / form 1 x 512 / form 0 x 768 threads:
@@ -525,7 +529,12 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
     }
     const bool mid = !driver && !large && slices <= (int64_t)4 * 8 * sms;
     const bool on_chip = mid && force_tpb == 0 && fmt == NN_FMT_SELL && a.ctl.cg_variant == 2 && mode != MODE_MIXED;
+    const char *sm_env = getenv("NNQP_SMEM_OP");
+    const bool smem_op = !(sm_env && sm_env[0] == '0');
+    const int64_t fours = (slices + 3) / 4;   // blocks of four slices
+    const bool few = slices <= (int64_t)4 * sms && (driver || o->grid_blocks <= 0 || o->grid_blocks >= fours);
     if (wide || (mid && (on_chip || slices > (int64_t)8 * sms / 2))) tpb = 512;
+    if (on_chip && few && smem_op) tpb = kSolveThreads;
     if (!driver && (force_tpb == 256 || force_tpb == 512)) tpb = force_tpb;
     if (large && (a.ctl.cg_variant == 0 || a.ctl.cg_variant == 3) && fmt == NN_FMT_SELL && force_tpb != 512)
         tpb = kLargeThreads;
@@ -561,19 +570,18 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
     // rather than filling fewer blocks' warps (measured: 40^3 transient on
     // 131 -> 152 blocks 55.8 -> 52.3 ms; 50^2 steady on 10 -> 19 blocks
     // 3.72 -> 3.36 ms)
-    const int64_t spread = on_chip && tpb == 512 ? slices : std::max<int64_t>(by_rows, (slices + 3) / 4);
+    const int64_t spread = on_chip && few ? fours : on_chip && tpb == 512 ? slices : std::max<int64_t>(by_rows, (slices + 3) / 4);
     int want = (int)std::min<int64_t>(spread, slices <= (int64_t)4 * 8 * sms ? (int64_t)sms : (int64_t)maxg);
     want = std::min(want, maxg);
     if (large) want = maxg;
     if (o->grid_blocks > 0) want = std::min(o->grid_blocks, maxg);
+    if (on_chip) want = std::min(want, sms);
     want = std::max(want, 1);
     // Mid-size SELL solves keep each block's slices of the operator of the
     // inner products in shared memory when they fit (one block per SM), and
     // the vectors of their pipelined CG phase (cg_resident.cuh).
     size_t dyn_smem = 0;
-    const char *sm_env = getenv("NNQP_SMEM_OP");
-    const bool smem_op = !(sm_env && sm_env[0] == '0');
-    if (!driver && fmt == NN_FMT_SELL && tpb == 512) {
+    if (!driver && fmt == NN_FMT_SELL && (tpb == 512 || (on_chip && few && tpb == 256))) {
         const int vbytes = mixed ? 4 : 8;
         const int64_t deep = (slices + want - 1) / want;   // slices of a block at most
         const int64_t most = block_entries(s, want);
@@ -599,7 +607,7 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
                 kern = ks;
                 dyn_smem = bytes;
                 maxg = per * sms;
-                a.ctl.res_warps = !resident ? 0 : rw ? std::min(atoi(rw), kResWarps) : resident_warps(deep);
+                a.ctl.res_warps = !resident ? 0 : rw ? std::min(atoi(rw), tpb == 512 ? kResWarps : 4) : resident_warps(deep);
                 a.res_offset = local ? (int)op : 0;
                 a.res_table = (int)table;
             }
@@ -607,20 +615,29 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
         cudaGetLastError();   // a refused attribute leaves the plain kernel in use
     }
     // Mid-size TRON (with Jacobi) and L-BFGS solves: the operator in shared
-    // memory, one block per SM as far as there are slices.  SSOR spreads its
-    // colours over all warps of a plain grid of 256-thread blocks: 512-thread
-    // blocks with the operator in shared memory are 1 to 6% slower alone (50 x 50
-    // 16.0 -> 17.1 ms, 30^3 68.5 -> 72.2) and half as many solves a second.
+    // memory, one block per SM as far as there are slices; small systems as above
+    // in blocks of four slices, TRON's of 256 threads.  L-BFGS blocks do not share
+    // an SM (216 registers a thread; 128 spill, 8 to 10% slower), so up to five
+    // slices to a block leave room for a second solve: 21 x 25 x 18 alone 7.3 ms
+    // with one block on every SM, 6.7 with 81 and with 65, and with four threads
+    // 128, 138 and 273 solves a second.  SSOR spreads its colours over all warps
+    // of a plain grid of 256-thread blocks: 512-thread blocks with the operator in
+    // shared memory are 1 to 6% slower alone (50 x 50 16.0 -> 17.1 ms, 30^3 68.5
+    // -> 72.2) and half as many solves a second.
     if (driver && !ssor && o->grid_blocks == 0 && slices <= (int64_t)4 * 8 * sms) {
-        const int w = (int)std::min<int64_t>(slices, sms);
+        const int64_t spread_lb = fours > sms / 2 && slices <= (int64_t)5 * (sms / 2) ? sms / 2 : fours;
+        const int w = (int)std::min<int64_t>(!few ? slices : lbfgs ? spread_lb : fours, sms);
         const int64_t deep = (slices + w - 1) / w;
         const size_t op = (size_t)deep * s->max_slice_slots * 12, table = ((size_t)(deep + 1) * 4 + 15) / 16 * 16;
         const size_t both = op + table + (size_t)kResVectors * deep * 32 * 8;
         const char *rw = getenv("NNQP_RES_WARPS");
         const bool res = tron && both <= kSmemBytes && !(rw && atoi(rw) < 1);
         const size_t bytes = res ? both : op;
-        GridKernel kt = res ? k_tron_grid<true, 512, true> : tron ? k_tron_grid<true, 512> : k_lbfgs_grid<true>;
-        const int t = tron ? 512 : kLbfgsThreads;
+        GridKernel kt = lbfgs        ? k_lbfgs_grid<true>
+                        : res && few ? k_tron_grid<true, kSolveThreads, true>
+                        : res        ? k_tron_grid<true, 512, true>
+                                     : k_tron_grid<true, 512>;
+        const int t = lbfgs ? kLbfgsThreads : res && few ? kSolveThreads : 512;
         if (op > 0 && op <= kSmemOperatorBytes &&
             cudaFuncSetAttribute((const void *)kt, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(res ? kSmemBytes : kSmemOperatorBytes)) == cudaSuccess) {

@@ -5,6 +5,7 @@ namespace nnqp {
 
 GridKernel grid_kernel_mixed_transient(int fmt, int cgv, int tpb) {
     if (fmt == FMT_SELL_SMEM_RES || fmt == FMT_SELL_RES) {
+        if (cgv == 2 && tpb == 256 && fmt == FMT_SELL_SMEM_RES) return k_solve_grid<4, MODE_MIXED_TR, 2, 256>;
         if (tpb != 512 || cgv != 2) return nullptr;
         return fmt == FMT_SELL_RES ? k_solve_grid<5, MODE_MIXED_TR, 2, 512> : k_solve_grid<4, MODE_MIXED_TR, 2, 512>;
     }
