@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
+#include <mutex>
 #include <vector>
 #include "../../include/nnqp.h"
 
@@ -134,6 +135,7 @@ struct nn_system {
     double *mdiag64 = nullptr;      // [NF]
     double *b0 = nullptr;           // [NF] F_F - K_FD c_D
     size_t assembly_peak_bytes = 0; // device bytes held at the end of assembly (system + temporaries)
+    std::mutex ssor_mu;             // held while the ordering is looked up and built
     nnqp::SsorF64 ssor{};           // SSOR ordering (ncolors = 0 until nn_precond_setup)
     int64_t ssor_slices = 0;
     std::vector<int32_t> ssor_color; // colour of each free unknown (host)

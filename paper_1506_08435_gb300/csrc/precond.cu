@@ -169,6 +169,8 @@ nn_status ssor_layout(int64_t n, int64_t ns, const int64_t *sptr, const int32_t 
 }
 
 nn_status ssor_setup(nn_system *s, cudaStream_t st) {
+    // (threads may make their first SSOR solves on one system together)
+    std::lock_guard<std::mutex> lk(s->ssor_mu);
     if (s->ssor.ncolors > 0) return NN_OK;
     const int64_t n = s->NF;
     if (n < 1) return NN_OK;   // nothing to order (no free unknowns)

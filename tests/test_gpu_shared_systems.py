@@ -18,6 +18,7 @@ THREADS = 8
 CASES = dict(step=(lambda: I.config2_transient_3d(n=9, nsteps=1), {}),
              square=(lambda: I.config1_steady_2d(n=30), {}),
              tron=(lambda: I.config1_steady_2d(n=30), dict(solver=P.NN_SOLVER_TRON)),
+             ssor=(lambda: I.config1_steady_2d(n=30), dict(precond=P.NN_PC_SSOR)),
              lbfgs=(lambda: I.config2_transient_3d(n=9, nsteps=1), dict(solver=P.NN_SOLVER_LBFGS)))
 
 
