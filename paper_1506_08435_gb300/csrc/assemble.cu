@@ -21,6 +21,7 @@
 #include "internal.h"
 #include "scan.cuh"
 #include "ops.cuh"
+#include "quotient.h"
 
 namespace nnqp {
 
@@ -214,20 +215,10 @@ __device__ __forceinline__ int tri_index(int a, int b, int nv) {  // a <= b, pac
     return a * nv - (a * (a - 1)) / 2 + (b - a);
 }
 
-// a / b, correctly rounded, from y = the correctly rounded 1 / b: one Newton
-// correction of the quotient by the exact remainder (P. Markstein, IBM J. Res.
-// Develop. 34, 1990).  Three operations, where a division is eight to ten; for
-// several quotients by one b.  b's magnitude is kept away from the ends of the
-// range by the callers.
-__device__ __forceinline__ double quotient(double a, double b, double y) {
-    const double q = __dmul_rn(a, y);
-    return fma(fma(-b, q, a), y, q);
-}
-
 // K_e (packed upper triangle, nv(nv+1)/2 values) and |e| of every element.
 // Bound by the FP64 pipe (a warp instruction holds a sub-core for 64 cycles),
 // so the operations are few, though every value is the same to the last bit as
-// from plain divisions: the nine quotients by det and |e| come from one
+// from plain divisions (quotient.h; cofactors between 2^-400 and 2^400): the nine quotients by det and |e| come from one
 // reciprocal, and the minors of D_e are formed only where they could be small.
 // 90 x 101 x 84 hexahedra, 4.6M tetrahedra: 2.62 -> 1.61 ms.  (1.06 ms with
 // K_ab = |e| (iso G_a.G_b + lon (v.G_a)(v.G_b)), whose last bits differ: they
@@ -471,7 +462,12 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_rows(int64_t N, const int32
                     x[u] = vol[e];
                     y[u] = a == b ? md : mo;
                 }
-                if (f_elem && l == 0) fr += quotient(__dmul_rn(f_elem[e], vol[e]), nv, 1.0 / nv);
+                if (f_elem && l == 0) {
+                    const double fe = __dmul_rn(f_elem[e], vol[e]);
+                    // (an infinite source stays what it is)
+                    const bool inf = (__double2hiint(fe) & 0x7ff00000) == 0x7ff00000;
+                    fr += inf ? fe : quotient(fe, nv, 1.0 / nv);
+                }
             }
         }
 #pragma unroll
