@@ -251,7 +251,7 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
     ctl.cg_max = 1 << 30;
     ctl.eta1 = kEta1;
     ctl.eta2 = kEta2;
-    ctl.from_afar = 0;   // (the batch has a cap of its own)
+    ctl.early_ratios = 0;   // (the batch has a cap of its own)
     ctl.mu = 1e-4;
     ctl.cg_variant = cgv;
     ctl.cg_bound_stop = 0;

@@ -266,7 +266,7 @@ struct GpcgCtl {
     // 0.1 for the second the cubes with a hole lose 5 to 18%, the others gain 3%.
     double eta1, eta2;
     double mu;           // Armijo constant
-    int from_afar;       // a steady solve with the early ratios (tightens the cap of the later refinements)
+    int early_ratios;    // eta1, eta2 are the early ones (tightens the cap of the later refinements)
     int cg_variant;      // 0: textbook PCG (3 team barriers per iteration);
                          // 1: Chronopoulos-Gear PCG (2 barriers, one fused reduction);
                          // 2: pipelined PCG (1 barrier: product, updates and

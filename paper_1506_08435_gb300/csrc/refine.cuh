@@ -14,34 +14,9 @@
 // FP64 KKT test; MixedStats::fallback records that this happened.
 #pragma once
 #include "gpcg.cuh"
+#include "inner_caps.h"
 
 namespace nnqp {
-
-// Products allowed to the first FP32 inner solve.  It starts from zero and
-// has to do most of the solve's work: CG needs O(sqrt(cond)) steps and cond
-// grows like n^(2/d), and GPCG adds the phases that find the active set
-// (steady solves of 5e4 - 1e6 unknowns from zero take 6k - 40k products).  A
-// cap only guards against an FP32 solve that cannot converge, so it is set
-// well above that: 64 sqrt(n), at least 4000.  Every later inner solve (a
-// correction of a residual already reduced) may take at most twice the
-// products of the first (a steady solve: 1,000 more than the first, below), so
-// a stagnating FP32 solve is cut off early and the contraction test then
-// hands the solve to FP64.
-__host__ __device__ __forceinline__ int64_t inner_product_cap(int64_t n) {
-    const int64_t c = (int64_t)(64.0 * sqrt((double)n));
-    return c > 4000 ? c : 4000;
-}
-
-// The same for the small instances of a batched solve (at most ~4e4
-// unknowns): 8 sqrt(n), at least 4000.  A capped inner solve there still
-// contracts the residual four-fold, and the refinement continues; with the
-// larger cap some FP32 inner solves ran long before converging (measured on
-// the 512-instance batch: 1.73M FP32 products and 275 solves/s against 1.63M
-// and 310 solves/s).
-__host__ __device__ __forceinline__ int64_t batch_inner_product_cap(int64_t n) {
-    const int64_t c = (int64_t)(8.0 * sqrt((double)n));
-    return c > 4000 ? c : 4000;
-}
 
 struct MixedStats {
     int64_t spmv64 = 0, spmv32 = 0, cg = 0, phases = 0, refinements = 0, vec64 = 0, vec32 = 0, fallback = 0;
@@ -152,14 +127,7 @@ __device__ int mixed_solve(Team &T, const Rows &R, const Op64 &A, const Op32 &A3
         Bounds<float> B{0.0, 0.0, l32, h32};
         int s = gpcg_call<SPLIT, Team, Op32, float, CGV32>(T, R, A32, B, v, c, is);
         if (ref == 0) {
-            // A later solve starts near its face and takes about half of the first
-            // with the early phase-end ratios (4,400 to 5,100, then 2,100 twice at
-            // 112 x 104 x 120).  One in some 25 there stalls in FP32 just above
-            // its tolerance, contracted by 7e3, and runs to the cap: with twice
-            // the first that solve took 15,058 products and 756 ms, so 11,617 and
-            // 583 ms (late ratios, whose first solve is twice as long: 619 ms).
-            const int64_t base = is.spmv > 1000 ? is.spmv : 1000;
-            const int64_t later = ctl32.from_afar ? base + 1000 : 2 * base;
+            const int64_t later = later_product_cap(is.spmv, ctl32.early_ratios != 0);
             if (later < inner_cap) inner_cap = later;
         }
         st.spmv32 += is.spmv;

@@ -425,7 +425,6 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
     const bool late = mode_transient(mode) || (force_tpb != 0 && s->dim == 3);
     a.ctl.eta1 = late ? kEta1Warm : kEta1;
     a.ctl.eta2 = late ? kEta2Warm : kEta2;
-    a.ctl.from_afar = !late;
     a.ctl.mu = 1e-4;
     // CG form: the pipelined one (one barrier per iteration) where barrier
     // latency bounds the solve; the textbook one on large systems, where the
@@ -457,6 +456,7 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
     if (const char *e = getenv("NNQP_GP_MAX")) a.ctl.gp_max = atoi(e);
     if (const char *e = getenv("NNQP_ETA1")) a.ctl.eta1 = atof(e);
     if (const char *e = getenv("NNQP_ETA2")) a.ctl.eta2 = atof(e);
+    a.ctl.early_ratios = a.ctl.eta1 >= kEta1 && a.ctl.eta2 >= kEta2;
     a.rtol = o->rtol;
     a.den_fallback = den_fallback(s);
     a.b0norm = s->b0norm;
