@@ -647,7 +647,8 @@ def run_batch(P, torch, args, rank):
     h2d = sum(nb for _, nb in hps) + sum(h.numel() * 8 for h in c0h)
     d2h = sum(h.numel() * 8 for h in outh)
     return dict(times=times, infos=infos, kern_ms=[o[0]["time_ms"] for o in outs],
-                kernel_name="k_batch_cluster" if tuned % 100 > 1 else "k_batch",
+                kernel_name="k_batch" if tuned % 100 == 1 else "k_batch_res" if tuned // 100 == 512 else
+                "k_batch_cluster",
                 kern_bytes=[sum(i["bytes_algo"] for i in o) for o in outs], units_per_step=count, e2e=e2e,
                 h2d=h2d, d2h=d2h, clocks=clocks, launches=launches,
                 sequential_fp64={"value": count / (seq_ms / 1e3), "unit": "QP solves/s", "ms": seq_ms,

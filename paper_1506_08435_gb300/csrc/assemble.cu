@@ -172,7 +172,7 @@ __device__ __forceinline__ bool inc_ok(int64_t m, int nv) { return m * nv <= kMa
 // Sorts every node's incidence list by (element, local vertex), so that all
 // later sums have one order, and counts its neighbours (the node itself among
 // them; an isolated node keeps its diagonal).  Bound by the scattered reads of
-// conn and the shared-memory atomics (L1 96% busy); 0.31 ms at the size above
+// conn and the shared-memory atomics; 0.31 ms at the size above
 // (sort 0.28 and count 0.69 before).
 template <int nv>
 __global__ void __launch_bounds__(kNodeBlock) k_node_count(int64_t N, const int32_t *__restrict__ conn,
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(TPB) k_element(int64_t E, const double *__rest
 // != 0 its row-sum lumping |e| delta_ab/(d+1).  Of a node's eight lanes, lane
 // b < nv adds vertex b's entry of K, lane 4 + b that of M (an element's
 // vertices differ, so no two lanes meet); eight incidences are fetched ahead of
-// their additions.  Bound by L1 (82%: the shared-memory sums); 0.75 ms at the
+// their additions.  Bound by L1 (the shared-memory sums); 0.75 ms at the
 // size above, where columns and sums took 0.69 + 1.20 ms.  Every sum is rounded
 // as one multiply-add per term in that order.
 template <int nv>

@@ -27,7 +27,8 @@ BatchKernel pick_kernel(bool mixed, int tpb, int cluster, int cgv) {
 // The default is 512 x 16.  A batch of 40 instances of 20 x 20 to 120 x 120
 // cells in FP64: one 256-thread block per instance (the former default) 590 ms,
 // bounded by the largest instance on one SM; clusters of 16 x 256 threads with
-// form 0 / 2 of CG 105 / 104 ms; this 61 ms.
+// form 0 / 2 of CG 105 / 104 ms; this 52 ms (with the same phase-end ratios; 38
+// with the early ones).
 struct BatchShape {
     int tpb = 512;
     int cluster = 16;
@@ -180,10 +181,12 @@ static nn_status run_batch(int count, nn_system *const *systems, double *const *
         launches.push_back({shape, false, 0, count, 0, 0});
     } else {
         // slices per CTA: what spreads the whole batch over the SMs, from 4 (a
-        // warp each) to 24 (three a warp).  Measured with 8 / 16 / 24 / 36: 40
-        // instances of 20 to 120 cells a side 66 / 60 / 63 / 61 ms, 20 mixed ones
-        // of 30 to 90 19.6 / 19.6 / 16.9 / 18.7 ms; 8 small ones of 20 to 50, which
-        // do not fill the device, 3.1 ms with 4 and 7.4 ms with 36.
+        // warp each) to 24 (three a warp).  Measured with 4 / 8 / 16 / 24 / 36: 40
+        // instances of 20 to 120 cells a side 46.3 / 44.4 / 42.0 / 42.8 / 39.0 ms
+        // and with other data 43.4 / 41.4 / 39.0 / 37.8 / 38.9; 20 mixed ones of 30
+        // to 90 15.7 / 14.1 / 14.0 / 11.0 / 12.9; 64 of 20 to 200 226 / 226 / 224 /
+        // 226 / 219; 8 small ones of 20 to 50, which do not fill the device, 3.1 /
+        // 3.4 / 4.3 / 5.5 / 6.8.
         int64_t total = 0;
         for (int i = 0; i < count; ++i) total += systems[i]->A64.nslices;
         const int64_t target = std::min<int64_t>(24, std::max<int64_t>(4, total / sms));

@@ -261,9 +261,13 @@ struct GpcgCtl {
     // late.  Products with (0.1, 1e-3) / (0.3, 0.06): 397 x 283 78,140 / 47,756,
     // 173 x 173 29,487 / 21,830, 120 x 120 11,456 / 7,502 (three problems each);
     // 44^3 15,146 / 10,679, 70^3 15,695 / 11,007, 90^3 mixed 20,360 / 14,705; 16
-    // batch instances 52,410 / 43,279; cube with a hole, m = 4 2,030 / 1,837 (m =
-    // 2 889 / 891, its 6% longer); 40^3 transient in time 19.7 / 20.3 ms.  With
+    // batch instances 52,410 / 43,279; cube with a hole, m = 4 2,030 / 1,837, m =
+    // 2 889 / 891; 40^3 transient in time 19.7 / 20.3 ms.  With
     // 0.1 for the second the cubes with a hole lose 5 to 18%, the others gain 3%.
+    // The kernels that only got the ratios, in time for three problems: CSR 50 x
+    // 50 21.3 / 17.7 ms, 397 x 283 920 / 568, 40^3 152 / 105, hole m = 2 6.3 / 6.1;
+    // SSOR 34.7 / 29.4, 1,119 / 731, 227 / 159, 12.9 / 13.1; mixed 23.5 / 20.9, 1,004 /
+    // 997 (its FP32 solves set its products), 132 / 91, 7.6 / 7.6.
     double eta1, eta2;
     double mu;           // Armijo constant
     int early_ratios;    // eta1, eta2 are the early ones (tightens the cap of the later refinements)

@@ -420,8 +420,11 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
     // need the long phases
     a.ctl.gp_max = mode_transient(mode) ? 3 : 50;
     a.ctl.cg_max = 1 << 30;
-    // (a served 3D solution, which the default tolerance leaves open by 1e-9, has
-    // to be the same bits from release to release: it keeps the late ratios)
+    // A served 3D request keeps the late ratios: at the default tolerance its
+    // solution is known to 1e-10 .. 2e-9 only (20 perturbed systems), the early
+    // ratios move it within that, and a server's answers were to stay where they
+    // were.  2D ones, known to some 1e-11, take the early ratios (their iterates and
+    // last bits are others than before), as nn_qp_solve does for both.
     const bool late = mode_transient(mode) || (force_tpb != 0 && s->dim == 3);
     a.ctl.eta1 = late ? kEta1Warm : kEta1;
     a.ctl.eta2 = late ? kEta2Warm : kEta2;
@@ -491,7 +494,8 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
     const int64_t slices = s->A64.nslices;
     int tpb = kSolveThreads;
     const bool driver = lbfgs || tron;   // solvers with a kernel of their own
-    // Large systems (more than 32 slices per SM) run one 768-thread block
+    // The largest systems (2^20 unknowns on; steady ones with more than 32
+    // slices per SM by the rule below) run one 768-thread block
     // per SM with the textbook CG form: the warps of three 256-thread blocks,
     // a third of the barrier arrivals and reduction partials.  (Served
     // requests of that size take the whole device, so they may too.)  Mixed
@@ -516,7 +520,11 @@ nn_status plan_build(nn_system *sys, const nn_solve_opts *o, int mode, int nstep
     // FP64 56^3 18.6 / 17.0 / 20.9, 72^3 32.4 / 27.5 / 32.1, 80^3 41.0 / 35.5 /
     // 38.9, 96^3 65.6 / 68.2 / 58.7; mixed (768 threads: the streamed FP32
     // operator, where it exceeds 48 MB) 56^3 18.7 / 12.7 / 17.8, 72^3 31.8 / 27.5 /
-    // 28.5, 80^3 32.0 / 29.6 / 28.1, 96^3 49.7 / 46.1 / 36.1.
+    // 28.5, 80^3 32.0 / 29.6 / 28.1, 96^3 49.7 / 46.1 / 36.1.  2D, with half the
+    // entries a row, crosses near the same sizes: FP64 420 x 390 15.3 / 12.3 /
+    // 17.1, 640 x 600 25.0 / 17.8 / 23.5, 800 x 720 33.6 / 31.2 / 29.4, 1000 x 900
+    // 49.1 / 48.7 / 41.9; mixed 17.1 / 11.3 / 14.8, 21.8 / 15.4 / 19.3, 30.2 / 19.3 /
+    // 23.7, 44.4 / 37.6 / 34.6.
     bool wide = false;   // one 512-thread block per SM
     if (large && !force_large && force_tpb == 0 && fmt == NN_FMT_SELL && a.ctl.cg_variant == 2 &&
         !mode_transient(mode) && !getenv("NNQP_CG_VARIANT")) {
