@@ -170,7 +170,7 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
     const double eta2 = C_.eta2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool compute = warp < na;
-    const int serve = (int)(blockDim.x >> 5) - 4;   // the first serving warp
+    constexpr int serve = IsResidentOp<Op>::threads / 32 - 4;   // the first serving warp
     RedSmem &sm = *in_shared(T.sm);
     const V zero = (V)0;
     const int ns = (int)(R.s1 - R.s0), nl = ns * 32, base = (int)(R.s0 * 32);
@@ -398,8 +398,8 @@ __device__ __noinline__ int cg_resident(Team &T_, const Rows &R_, const Op &A_, 
                     al = an;
                     if (ss + an * (2.0 * sp + an * pp) >= tr->dd) {
                         out = 1.0;
-                        const double h = sp / pp;                  // (not sp^2, for the same reason)
-                        tau = sqrt(fmax(h * h + (tr->dd - ss) / pp, 0.0)) - h;
+                        const double ip = 1.0 / pp, h = sp * ip;   // (not sp^2, for the same reason)
+                        tau = sqrt(fmax(fma(h, h, (tr->dd - ss) * ip), 0.0)) - h;
                     }
                 }
                 if (lane == 0) {

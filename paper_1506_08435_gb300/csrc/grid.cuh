@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : FMT >= 4 ? 2 : mode_min_
             }
             MixedStats ms;
             if constexpr (RES) {
-                SellF32DiffResX<LOCAL> A32r;
+                SellF32DiffResX<LOCAL, TPB> A32r;
                 if constexpr (LOCAL) static_cast<SellF32DiffLocal &>(A32r) = A32loc;
                 else static_cast<SellF32Diff &>(A32r) = a.A32;
                 status = mixed_solve<CGV, inner_cg_form(MODE, CGV), true>(T, R, a.A, A32r, a.lo, a.hi, b, x, v, a.v32[9], a.v32[10],
@@ -280,10 +280,10 @@ __global__ void __launch_bounds__(TPB, TPB >= 512 ? 1 : FMT >= 4 ? 2 : mode_min_
             GpcgStats gs;
             const Bounds<double> B{a.lo, a.hi, nullptr, nullptr};
             if constexpr (RES) {
-                SellF64ResX<LOCAL> Ar;
+                SellF64ResX<LOCAL, TPB> Ar;
                 if constexpr (LOCAL) static_cast<SellF64Local &>(Ar) = Aloc;
                 else static_cast<SellF64 &>(Ar) = a.A;
-                status = gpcg_solve<GridTeam, SellF64ResX<LOCAL>, double, CGV>(T, R, Ar, B, v, c, gs);
+                status = gpcg_solve<GridTeam, SellF64ResX<LOCAL, TPB>, double, CGV>(T, R, Ar, B, v, c, gs);
             } else if constexpr (FMT == 0)
                 status = gpcg_solve<GridTeam, SellF64, double, CGV>(T, R, a.A, B, v, c, gs);
             else if constexpr (LOCAL)

@@ -399,22 +399,24 @@ struct SellF32DiffTma {
 // The same operators by another type, for the kernels whose CG phase keeps its
 // vectors in shared memory (cg_resident.cuh): in shared memory themselves or
 // read from global memory (the same entries in the same order: the results are
-// the same bits).
-template <bool LOCAL>
+// the same bits), in blocks of TPB threads.
+template <bool LOCAL, int TPB = 512>
 struct SellF64ResX : SellF64X<LOCAL> {};
-template <bool LOCAL>
+template <bool LOCAL, int TPB = 512>
 struct SellF32DiffResX : SellF32DiffX<LOCAL> {};
 template <class Op>
 struct IsResidentOp {
     static constexpr bool value = false;
 };
-template <bool L>
-struct IsResidentOp<SellF64ResX<L>> {
+template <bool L, int TPB>
+struct IsResidentOp<SellF64ResX<L, TPB>> {
     static constexpr bool value = true, local = L;
+    static constexpr int threads = TPB;
 };
-template <bool L>
-struct IsResidentOp<SellF32DiffResX<L>> {
+template <bool L, int TPB>
+struct IsResidentOp<SellF32DiffResX<L, TPB>> {
     static constexpr bool value = true, local = L;
+    static constexpr int threads = TPB;
 };
 
 // Whether an operator streams through L2 (large systems): the vector passes
@@ -423,10 +425,10 @@ template <bool L>
 __device__ __forceinline__ bool op_streams(const SellF64X<L> &A) { return A.stream; }
 template <bool L>
 __device__ __forceinline__ bool op_streams(const SellF32DiffX<L> &A) { return A.stream; }
-template <bool L>
-__device__ __forceinline__ bool op_streams(const SellF64ResX<L> &A) { return A.stream; }
-template <bool L>
-__device__ __forceinline__ bool op_streams(const SellF32DiffResX<L> &A) { return A.stream; }
+template <bool L, int TPB>
+__device__ __forceinline__ bool op_streams(const SellF64ResX<L, TPB> &A) { return A.stream; }
+template <bool L, int TPB>
+__device__ __forceinline__ bool op_streams(const SellF32DiffResX<L, TPB> &A) { return A.stream; }
 __device__ __forceinline__ bool op_streams(const SellF32DiffTma &) { return true; }
 template <class Op>
 __device__ __forceinline__ bool op_streams(const Op &) { return false; }

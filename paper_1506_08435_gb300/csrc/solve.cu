@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(TPB, LOCAL && TPB == 512 ? 1 : 2) k_tron_grid(
     const Rows R = rows_of_block(a.n, a.nslices, blockIdx.x, gridDim.x);
     T.active = a.pc.ncolors > 0 ? (int)(blockDim.x >> 5) : R.active_warps(blockDim.x >> 5);
     static_assert(!RES || LOCAL, "the resident kernel has its operator in shared memory");
-    std::conditional_t<RES, SellF64ResX<LOCAL>, SellF64X<LOCAL>> A;
+    std::conditional_t<RES, SellF64ResX<LOCAL, TPB>, SellF64X<LOCAL>> A;
     if constexpr (LOCAL) static_cast<SellF64Local &>(A) = stage_operator(a.A, R, drv_smem);
     else A = a.A;
     double *x0 = a.v64[0];
